@@ -104,7 +104,7 @@ def draw(rng):
     elif kind == "precond":
         c = _case("", "precond", _dims(rng, 256, 1 << 20), prec=rng.choice(["fp16", "fp16", "fp32"]))
     else:
-        c = _case("", "grad", _dims(rng, 1 << 10, 1 << 17), samples=rng.choice([1, 2, 4]))
+        c = _case("", "grad", _dims(rng, 1 << 17, 5 << 16), samples=rng.choice([4, 6, 8]))
     del c["name"]
     return c
 
@@ -192,6 +192,7 @@ def prepare(case, seed):
             s["out_" + prec] = torch.empty_like(s[prec])
         return s
     lat = _lattice(case, u)
+    links = u if kind == "grad" else None
     del u
     s = {"case": case, "lat": lat}
     if kind == "apply":
@@ -209,16 +210,22 @@ def prepare(case, seed):
         run(s)
     else:
         lat.precond_set(_weights(seed))
-        v, y = _samples(case, seed)
+        v, y = _samples(case, seed, links)
         s["v"] = _packed(lat, "fp32", [0], v).flatten(1)
         s["y"] = _packed(lat, "fp32", [0], y).flatten(1)
     return s
 
 
-def _samples(case, seed):
-    """Training pairs: Gaussian v, and y = v plus a part of its own (A^-1 v is v to first order)."""
+def _samples(case, seed, u):
+    """Training pairs: Gaussian v, and y = v + K v + K K v, K = kappa^2 H_eo H_oe, which A^-1 v is to second order."""
     v = _fields(case, seed, case["samples"])
-    return v, v + 0.3 * _fields(case, seed, case["samples"], 4)
+    y = v.clone()
+    for i in range(case["samples"]):
+        f = _on(torch.view_as_complex(v[i]), _size(case), 0)
+        for _ in range(2):
+            f = case["kappa"] ** 2 * _hop(u, _hop(u, f))
+            y[i] += torch.view_as_real(f)
+    return v, y
 
 
 def run(s):
@@ -243,7 +250,7 @@ def run(s):
         lat.precond_apply(case["prec"], s["in"], s["out"])
         return s["out"]
     loss, grad = lat.precond_grad(s["v"], s["y"], 1.0)
-    return [loss, grad]
+    return [torch.tensor(loss, dtype=torch.float32), grad]
 
 
 # --- what a pass cannot do without ----------------------------------------------------------------------------------
@@ -455,7 +462,7 @@ def exact(case, seed):
         for c in range(C_MID):      # one hidden channel at a time
             out += _layer(u, w2[:, None, c:c + 1], _layer(u, w1[:, c:c + 1, None], f[None]))[0]
         return _lay(case, out, case["prec"], [0])[None]
-    v, y = _samples(case, seed)
+    v, y = _samples(case, seed, u)
     total, grad, k = 0.0, torch.zeros_like(w), case["kappa"]
     for i in range(case["samples"]):
         a, b = (_on(_stored(q[i], "fp32"), dims, 0) for q in (v, y))
