@@ -51,6 +51,9 @@ int num_sms() {
     return n;
 }
 
+// Largest deviation of U U^+ from 1 and of det U from 1 of links taken as SU(3).
+constexpr double SU3_DEV = 1e-6;
+
 static int prec_bytes(int prec) { return prec == WD_FP64 ? 8 : prec == WD_FP32 ? 4 : 2; }
 int link_units(int prec, int recon) { return 8 * recon * prec_bytes(prec) / 16; }
 int spinor_units(int prec) { return 24 * prec_bytes(prec) / 16; }
@@ -137,7 +140,7 @@ int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const ui
     if (!valid_prec(prec) || !valid_recon(recon)) return fail(h, WD_ERR_INVALID_ARG, "bad precision %d or recon %d", prec, recon);
     const int ri = recon == 12 ? 0 : 1;
     if (!h->links[prec][ri][0]) {
-        if (recon == 12 && (h->unit_dev > 1e-6 || h->det_dev > 1e-6))
+        if (recon == 12 && (h->unit_dev > SU3_DEV || h->det_dev > SU3_DEV))
             return fail(h, WD_ERR_NOT_SU3, "12-real links need SU(3) links: max |UU^+ - 1| = %g, max |det U - 1| = %g",
                         h->unit_dev, h->det_dev);
         const size_t bytes = (size_t)h->g.Vh * link_units(prec, recon) * 16;
@@ -147,7 +150,7 @@ int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const ui
             h->links[prec][ri][p] = buf;
             cudaError_t e = by_prec(prec, [&](auto tag) {
                 typedef typename decltype(tag)::type T;
-                return Ops<T>::build_links(recon, h->g, p, h->U64, buf, 0);
+                return Ops<T>::build_links(recon, h->g, p, h->U64, buf, h->fixed64, 0);
             });
             if (e != cudaSuccess) return cuda_fail(h, e, "build_links");
         }
@@ -308,6 +311,12 @@ int wd_set_gauge(wd_handle* h, const double* U, int where) {
     WD_CUDA(h, cudaMemcpy(host, dev, sizeof host, cudaMemcpyDeviceToHost));
     std::memcpy(&h->unit_dev, &host[0], sizeof(double));
     std::memcpy(&h->det_dev, &host[1], sizeof(double));
+    // SU(3) links (the 12-real criterion) let the FP64 hop run in fixed point
+    const bool fixed64 = h->unit_dev <= SU3_DEV && h->det_dev <= SU3_DEV;
+    if (fixed64 != h->fixed64) {
+        h->fixed64 = fixed64;
+        h->gen += 1;   // captured solver graphs hold the other kernels
+    }
     h->have_gauge = true;
     if (h->have_clover) return clover_build(h);   // the clover blocks follow the links
     return WD_OK;

@@ -7,6 +7,7 @@
 
 #include <cstring>
 
+#include "fixed64.cuh"
 #include "kernels.h"
 
 namespace wd {
@@ -660,7 +661,8 @@ __global__ void k_unpack(Geom g, int parity, const uint4* in, double* lex) {
 }
 
 // Gathered links of output parity p (see hop_impl.cuh) from FP64 lex links.
-template <typename T, int R>
+// FIXED: every FP64 real as its two fixed-point digits (fixed64.cuh).
+template <typename T, int R, bool FIXED>
 __global__ void k_build_links(Geom g, int parity, const double* U, uint4* out) {
     constexpr int N = Unit<T>::N;
     const int V = 2 * g.Vh;
@@ -687,8 +689,18 @@ __global__ void k_build_links(Geom g, int parity, const double* U, uint4* out) {
                 const double vf = zf ? 0.0 : uf[e];
                 const double vb = zb ? 0.0 : (im ? -ub[2 * (3 * b + a) + 1] : ub[2 * (3 * b + a)]);
                 const int ef = (2 * mu) * R + e, eb = (2 * mu + 1) * R + e;
-                reinterpret_cast<T*>(out + (size_t)(ef / N) * g.Vh + h)[ef % N] = from_double<T>(vf);
-                reinterpret_cast<T*>(out + (size_t)(eb / N) * g.Vh + h)[eb % N] = from_double<T>(vb);
+                T* const of = reinterpret_cast<T*>(out + (size_t)(ef / N) * g.Vh + h) + ef % N;
+                T* const ob = reinterpret_cast<T*>(out + (size_t)(eb / N) * g.Vh + h) + eb % N;
+                if constexpr (FIXED) {
+                    int2 wf, wb;
+                    fx::link_digits(vf, wf.x, wf.y);
+                    fx::link_digits(vb, wb.x, wb.y);
+                    *reinterpret_cast<int2*>(of) = wf;
+                    *reinterpret_cast<int2*>(ob) = wb;
+                } else {
+                    *of = from_double<T>(vf);
+                    *ob = from_double<T>(vb);
+                }
             }
         }
     }

@@ -38,6 +38,7 @@ struct wd_handle {
     double* U64 = nullptr;             // FP64 links, host layout, on the device
     bool have_gauge = false;
     double unit_dev = -1.0, det_dev = -1.0;
+    bool fixed64 = false;              // the FP64 18-real links are held as fixed-point digits (SU(3) links)
     uint4* links[4][2][2] = {};        // [prec][recon 12 -> 0, 18 -> 1][output parity]
 
     std::map<std::string, Buffer> ws; // named device workspaces
@@ -104,6 +105,7 @@ inline void apply_tuning(const wd_handle* h, int prec, int recon, HopParams& P) 
         P.block[f] = h->tune_block[prec][recon == 12 ? 0 : 1][f];
     }
     P.arith16 = (prec == WD_FP16 && h->arith16) ? 1 : 0;
+    P.fixed64 = (prec == WD_FP64 && recon == 18 && h->fixed64) ? 1 : 0;
     P.wait_rounds = h->wait_rounds;
     for (int f = 0; f < 2; ++f) {
         P.rhs_group[f] = P.arith16 ? h->tune_rhs[recon == 12 ? 0 : 1][f] : 0;

@@ -44,6 +44,7 @@ struct HopParams {
     int rhs_group[2];          // FP16 arithmetic: right-hand sides per thread (hop16m_kernel) without / with a
                                // fused reduction; 0 or 1 = one (hop16_kernel); must divide nrhs to be used
     int rhs_smem[2];           // ... and 1 = the site's links in shared memory instead of registers
+    int fixed64;               // FP64, 18-real: the links are fixed-point digits (hop64_kernel)
     int spt;                   // FP16 arithmetic, plain hop: sites per thread (grid-stride; 0 or 1 = one site)
 };
 
@@ -92,7 +93,9 @@ template <typename T> struct Ops {
     static cudaError_t chiral_from64(int n, const uint4* src64, uint4* dst, cudaStream_t s);
     static cudaError_t pack(const Geom& g, int parity, const double* lex, uint4* out, cudaStream_t s);
     static cudaError_t unpack(const Geom& g, int parity, const uint4* in, double* lex, cudaStream_t s);
-    static cudaError_t build_links(int recon, const Geom& g, int parity, const double* U, uint4* out, cudaStream_t s);
+    // fixed64: FP64 18-real links as fixed-point digits (SU(3) links only; fixed64.cuh)
+    static cudaError_t build_links(int recon, const Geom& g, int parity, const double* U, uint4* out, bool fixed64,
+                                   cudaStream_t s);
 };
 
 cudaError_t launch_unitarity(int nlinks, const double* U, unsigned long long* out, cudaStream_t s);

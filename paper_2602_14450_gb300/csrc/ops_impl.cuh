@@ -12,6 +12,7 @@
 #include "hop16_impl.cuh"
 #include "hop16m_impl.cuh"
 #include "hop3_impl.cuh"
+#include "hop64_impl.cuh"
 #include "hop_impl.cuh"
 #include "kernels.h"
 
@@ -121,6 +122,18 @@ cudaError_t run_hop16m(const HopParams& Q, int K, cudaStream_t s) {
     return launch_k(hop16m_kernel<R, E, D, LSM>, nb * groups, blk, smem, s, Q);
 }
 
+// The FP64 hop in fixed point (SU(3) links). wd_tune's block size applies up to the kernel's 128 threads; the
+// kernel variants are those of the floating-point hop and do not.
+template <int E, int D, bool MAT>
+cudaError_t run_hop64(const HopParams& P, cudaStream_t s) {
+    constexpr int form = D == RED_NONE ? 0 : 1;
+    const int block = P.block[form] > 0 && P.block[form] < HOP64_THREADS ? P.block[form] : HOP64_THREADS;
+    const void* k = (const void*)hop64_kernel<E, D, MAT>;
+    const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, block) : reduce_blocks(k, P.g.Vh, block, P.nrhs);
+    const cudaError_t e = launch_k(hop64_kernel<E, D, MAT>, nb * P.nrhs, block, 0, s, P);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <typename T, int R, int E, int D>
 cudaError_t run_hop(const HopParams& P, cudaStream_t s) {
     if constexpr (std::is_same<T, __half>::value) {
@@ -155,6 +168,9 @@ cudaError_t run_hop(const HopParams& P, cudaStream_t s) {
             }
             return cudaGetLastError();
         }
+    }
+    if constexpr (std::is_same<T, double>::value && R == 18) {
+        if (P.fixed64) return P.mat ? run_hop64<E, D, true>(P, s) : run_hop64<E, D, false>(P, s);
     }
     if (P.mat) {   // with a site-local block (clover): the one-site-per-thread look-ahead kernel
         const int blk = 128;
@@ -361,11 +377,14 @@ cudaError_t Ops<T>::unpack(const Geom& g, int parity, const uint4* in, double* l
 }
 
 template <typename T>
-cudaError_t Ops<T>::build_links(int recon, const Geom& g, int parity, const double* U, uint4* out, cudaStream_t s) {
+cudaError_t Ops<T>::build_links(int recon, const Geom& g, int parity, const double* U, uint4* out, bool fixed64,
+                                cudaStream_t s) {
     if (recon == 12)
-        k_build_links<T, 12><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
+        k_build_links<T, 12, false><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
+    else if (recon == 18 && fixed64 && std::is_same<T, double>::value)
+        k_build_links<T, 18, true><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
     else if (recon == 18)
-        k_build_links<T, 18><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
+        k_build_links<T, 18, false><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
