@@ -15,8 +15,13 @@ namespace wd {
 // out = (a + ib) * v for one complex element pair
 template <typename C>
 __device__ __forceinline__ void cscale_add(C& or_, C& oi, C ar, C ai, C vr, C vi) {
-    or_ += ar * vr - ai * vi;
-    oi += ar * vi + ai * vr;
+    if constexpr (sizeof(C) == 8) {   // two FP64 operations each instead of three
+        or_ = fma(-ai, vi, fma(ar, vr, or_));
+        oi = fma(ai, vr, fma(ar, vi, oi));
+    } else {
+        or_ += ar * vr - ai * vi;
+        oi += ar * vi + ai * vr;
+    }
 }
 
 #define GRID_STRIDE(h, n) for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < (n); h += gridDim.x * blockDim.x)
@@ -244,8 +249,8 @@ __global__ void __launch_bounds__(256) k_xr(int n, int nrhs, long long vs, uint4
 #pragma unroll
                     for (int i = 0; i < ST::N / 2; ++i) {
                         const C rsr = Unit<T>::get(urs[c], 2 * i), rsi = Unit<T>::get(urs[c], 2 * i + 1);
-                        s_re += rsr * rr[2 * i] + rsi * rr[2 * i + 1];
-                        s_im += rsr * rr[2 * i + 1] - rsi * rr[2 * i];
+                        add_products(s_re, rsr, rr[2 * i], rsi, rr[2 * i + 1]);
+                        sub_products(s_im, rsr, rr[2 * i + 1], rsi, rr[2 * i]);
                     }
                 }
             }
@@ -280,9 +285,9 @@ __global__ void __launch_bounds__(256) k_scale(int n, int nrhs, long long vs, ui
         load_spinor<T>(rstar, n, h, rs);
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
-            s_r2 += rr[2 * i] * rr[2 * i] + rr[2 * i + 1] * rr[2 * i + 1];
-            s_re += rs[2 * i] * rr[2 * i] + rs[2 * i + 1] * rr[2 * i + 1];
-            s_im += rs[2 * i] * rr[2 * i + 1] - rs[2 * i + 1] * rr[2 * i];
+            add_products(s_r2, rr[2 * i], rr[2 * i], rr[2 * i + 1], rr[2 * i + 1]);
+            add_products(s_re, rs[2 * i], rr[2 * i], rs[2 * i + 1], rr[2 * i + 1]);
+            sub_products(s_im, rs[2 * i], rr[2 * i + 1], rs[2 * i + 1], rr[2 * i]);
         }
         if (resx) {
             C xx[24];

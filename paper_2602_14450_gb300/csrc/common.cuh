@@ -709,34 +709,55 @@ __device__ __forceinline__ Slice slice_of(int nrhs) {
     return s;
 }
 
+// Sums of FP64 values. The FP64 pipe takes 64 cycles per warp instruction (half a lane per cycle and SM
+// sub-partition), so the sums are folded instead of reduced one after the other: exchanging with the lane 16
+// away, a lane keeps half of the sums, then with the lane 8 away a quarter, and the last steps add one value per
+// lane -- 6 additions per warp for four sums, where a shuffle tree per sum takes 20. Sum k ends in the lanes
+// k * 32 / P .. (P = NSUM rounded up to a power of two).
+template <int NSUM> struct FoldedSums {
+    static constexpr int P = NSUM <= 1 ? 1 : NSUM <= 2 ? 2 : 4;
+    static_assert(NSUM <= 4, "at most four sums");
+};
 template <int NSUM>
-__device__ __forceinline__ void warp_sum(double (&v)[NSUM]) {
+__device__ __forceinline__ double warp_fold(const double (&v)[NSUM]) {
+    constexpr int P = FoldedSums<NSUM>::P;
+    const int lane = threadIdx.x & 31;
+    double w[P];
 #pragma unroll
-    for (int k = 0; k < NSUM; ++k) {
+    for (int k = 0; k < P; ++k) w[k] = k < NSUM ? v[k < NSUM ? k : 0] : 0.0;
+    int off = 16;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
+    for (int n = P; n > 1; n >>= 1, off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int k = 0; k < n / 2; ++k) {
+            const double mine = up ? w[k + n / 2] : w[k], theirs = up ? w[k] : w[k + n / 2];
+            w[k] = mine + __shfl_xor_sync(0xffffffffu, theirs, off);
+        }
     }
+    double r = w[0];
+    for (; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    return r;
 }
 
-// Sum v over the block; the result is valid in thread 0. FP64 additions are
-// slow on this GPU (64 cycles of latency each), so the second level adds the
-// few warp sums one after the other instead of another five-step shuffle.
+// Sum v over the block; the result is valid in thread 0. Lane k of warp 0 adds the warps' shares of sum k.
 template <int NSUM>
 __device__ __forceinline__ void block_sum(double (&v)[NSUM]) {
+    constexpr int P = FoldedSums<NSUM>::P;
     __shared__ double sh[NSUM][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    warp_sum<NSUM>(v);
+    const double r = warp_fold<NSUM>(v);
     __syncthreads();   // sh may still be read by a previous call
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < NSUM; ++k) sh[k][warp] = v[k];
-    }
+    if ((lane & (32 / P - 1)) == 0 && lane / (32 / P) < NSUM) sh[lane / (32 / P)][warp] = r;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < nw; ++w) {
-#pragma unroll
-            for (int k = 0; k < NSUM; ++k) v[k] += sh[k][w];
+    if (warp == 0) {
+        double t = 0.0;
+        if (lane < NSUM) {
+            t = sh[lane][0];
+            for (int w = 1; w < nw; ++w) t += sh[lane][w];
         }
+#pragma unroll
+        for (int k = 0; k < NSUM; ++k) v[k] = __shfl_sync(0xffffffffu, t, k);
     }
 }
 
@@ -753,7 +774,7 @@ __device__ __forceinline__ unsigned ticket_add(unsigned* t) {
 
 // Reduce v over the sl.nb blocks that serve right-hand side sl.rhs (HINT: the
 // scalar stage the calling kernel expects to run). The last block adds the partial sums with all its threads (each thread loads its
-// eight next partials before adding them, so the loads overlap), then sums
+// four next partials before adding them, so the loads overlap), then sums
 // over the block; FP64 arithmetic is shared by the SM's warps, so spreading it
 // over the block's warps matters more than its latency.
 template <int NSUM, int HINT = ST_NONE>
@@ -782,18 +803,20 @@ __device__ __forceinline__ void grid_reduce(const double (&vin)[NSUM], const Red
 #pragma unroll
     for (int k = 0; k < NSUM; ++k) acc[k] = 0.0;
     const int nt = blockDim.x;
-    for (int b0 = threadIdx.x; b0 < sl.nb; b0 += 8 * nt) {
-        double t[8][NSUM];
+    for (int b0 = threadIdx.x; b0 < sl.nb; b0 += 4 * nt) {
+        double t[4][NSUM];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 4; ++i) {
             const int b = b0 + i * nt;
 #pragma unroll
             for (int k = 0; k < NSUM; ++k) t[i][k] = b < sl.nb ? __ldcg(part + (size_t)b * NSUM + k) : 0.0;
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < 4; ++i) {
+            if ((b0 - (int)threadIdx.x) + i * nt >= sl.nb) break;   // no thread of the block has a partial sum left
 #pragma unroll
             for (int k = 0; k < NSUM; ++k) acc[k] += t[i][k];
+        }
     }
     WD_TL_T(5)
     block_sum<NSUM>(acc);

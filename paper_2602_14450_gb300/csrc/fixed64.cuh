@@ -15,7 +15,7 @@
 //
 // Errors, in units of 2^(E-1078), at most 2^-55 of the largest neighbour real:
 // a product of a link row with a column is off by at most 3.5 (spinor reals cut
-// at 1/8 each: 0.6; u0 h0 left out: 1.5; link entries: 0.4; its own rounding
+// at 1/8 each: 0.6; u0 h0 left out: 1.5; link entries: 0.2; its own rounding
 // and a shift: 1), typically 0.3, and a site's sum is rounded once more to
 // FP64. The relative error of a hop of Gaussian fields is 0.92e-16 against
 // 1.0e-16 in FP64 arithmetic (~25 roundings at 2^-53).
@@ -55,7 +55,11 @@ __host__ __device__ __forceinline__ unsigned long long shr64(unsigned long long 
 // The 64-bit fixed-point link entry of a double in [-1.001, 1.001] as (u0, u1): both digits may be negated.
 __host__ __device__ __forceinline__ void link_digits(double u, int& u0, int& u1) {
     const double s = u * 2305843009213693952.0;   // 2^61
-    long long v = (long long)s;
+#ifdef __CUDA_ARCH__
+    long long v = __double2ll_rn(s);
+#else
+    long long v = llrint(s);
+#endif
     int lo = (int)(unsigned)(unsigned long long)v;
     if (lo == (int)0x80000000) {                  // -2^31 has no negative: move the entry by one unit
         v += 1;

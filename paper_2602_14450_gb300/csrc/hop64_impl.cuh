@@ -78,7 +78,9 @@ __device__ __forceinline__ void rebuild_fixed(int mu, bool fwd, const long long 
 }
 
 constexpr int HOP64_THREADS = 128;
-constexpr int HOP64_BLOCKS = 3;   // per SM: 168 registers; 4 (128 registers, spills) 435 against 425 us
+// Resident blocks per SM: 4 (128 registers). 3 (168 registers) is 2% faster at 32^3 x 64 (425 against 435 us), but at
+// 16^3 x 32 it leaves 56 of the 512 blocks to a second wave.
+constexpr int HOP64_BLOCKS = 4;
 
 // Bounds: a warp issues about 7500 instructions per 32 sites, 1728 of them
 // wide integer multiply-adds, which occupy the multiplier pipe 4.4-5.7 cycles

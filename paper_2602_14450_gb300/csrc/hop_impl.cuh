@@ -233,16 +233,25 @@ __device__ __forceinline__ void hop_epilogue(const HopParams& P, uint4* vout, co
 #pragma unroll
     for (int i = 0; i < 24; ++i) o[i] = (EPI == EPI_H && P.a == 1.0) ? acc[i] : ca * acc[i];
     C yv[24];
+    [[maybe_unused]] const bool unit_b = P.b == 1.0;
     if constexpr (EPI >= EPI_Y) {
         load_spinor<T>(vy, Vh, h, yv);
 #pragma unroll
-        for (int i = 0; i < 24; ++i) o[i] += cb * yv[i];
+        for (int i = 0; i < 24; ++i) {
+            // FP64, b = 1 (the even-odd operator, D_W and the residual): one operation per real instead of two
+            if (sizeof(C) == 8 && unit_b) o[i] = fma(ca, acc[i], yv[i]);
+            else o[i] += cb * yv[i];
+        }
     }
     if constexpr (EPI >= EPI_YZ) {
         C zv[24];
         load_spinor<T>(vz, Vh, h, zv);
 #pragma unroll
-        for (int i = 0; i < 24; ++i) o[i] += cc * zv[i];
+        for (int i = 0; i < 24; ++i) {
+            // FP64 residual r = (y - x) + a H: the two large terms are subtracted before the small one is added
+            if (sizeof(C) == 8 && unit_b && P.c == -1.0) o[i] = fma(ca, acc[i], yv[i] - zv[i]);
+            else o[i] += cc * zv[i];
+        }
     }
     store_spinor<T>(vout, Vh, h, o, ftz);
 
@@ -251,8 +260,8 @@ __device__ __forceinline__ void hop_epilogue(const HopParams& P, uint4* vout, co
         load_spinor<T>(vrs, Vh, h, rs);
 #pragma unroll
         for (int i = 0; i < 12; ++i) {   // conj(rs) * o
-            part[0] += rs[2 * i] * o[2 * i] + rs[2 * i + 1] * o[2 * i + 1];
-            part[1] += rs[2 * i] * o[2 * i + 1] - rs[2 * i + 1] * o[2 * i];
+            add_products(part[0], rs[2 * i], o[2 * i], rs[2 * i + 1], o[2 * i + 1]);
+            sub_products(part[1], rs[2 * i], o[2 * i + 1], rs[2 * i + 1], o[2 * i]);
         }
     } else if constexpr (RED == RED_TS) {          // (o, q), (o, o), (q, q); q = rstar if given, else y
         C qv[24];
@@ -264,10 +273,10 @@ __device__ __forceinline__ void hop_epilogue(const HopParams& P, uint4* vout, co
         }
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
-            part[0] += o[2 * i] * qv[2 * i] + o[2 * i + 1] * qv[2 * i + 1];
-            part[1] += o[2 * i] * qv[2 * i + 1] - o[2 * i + 1] * qv[2 * i];
-            part[2] += o[2 * i] * o[2 * i] + o[2 * i + 1] * o[2 * i + 1];
-            part[NS - 1] += qv[2 * i] * qv[2 * i] + qv[2 * i + 1] * qv[2 * i + 1];
+            add_products(part[0], o[2 * i], qv[2 * i], o[2 * i + 1], qv[2 * i + 1]);
+            sub_products(part[1], o[2 * i], qv[2 * i + 1], o[2 * i + 1], qv[2 * i]);
+            add_products(part[2], o[2 * i], o[2 * i], o[2 * i + 1], o[2 * i + 1]);
+            add_products(part[NS - 1], qv[2 * i], qv[2 * i], qv[2 * i + 1], qv[2 * i + 1]);
         }
     } else if constexpr (RED == RED_NORM) {
 #pragma unroll
