@@ -76,6 +76,14 @@ inline int stream_blocks(int n, int block) {
     return g < 1 ? 1 : (int)g;
 }
 
+// Threads per block of a launch over n items for each of nrhs right-hand sides: `block`, or on a small lattice a
+// half, quarter, ... of it down to one warp until every SM has a block. A kernel of 16 blocks of 128 threads (8^4)
+// otherwise runs on 16 of the 152 SMs.
+inline int spread_block(int n, int nrhs, int block) {
+    while (block > 32 && (long)stream_blocks(n, block) * nrhs < num_sms()) block /= 2;
+    return block;
+}
+
 // Tiling of the staged hop kernel, or false when its shared memory would not
 // allow two resident blocks per SM.
 template <typename T, int R>
@@ -127,7 +135,8 @@ cudaError_t run_hop16m(const HopParams& Q, int K, cudaStream_t s) {
 template <int E, int D, bool MAT>
 cudaError_t run_hop64(const HopParams& P, cudaStream_t s) {
     constexpr int form = D == RED_NONE ? 0 : 1;
-    const int block = P.block[form] > 0 && P.block[form] < HOP64_THREADS ? P.block[form] : HOP64_THREADS;
+    const int block = spread_block(P.g.Vh, P.nrhs, P.block[form] > 0 && P.block[form] < HOP64_THREADS
+                                                       ? P.block[form] : HOP64_THREADS);
     const void* k = (const void*)hop64_kernel<E, D, MAT>;
     const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, block) : reduce_blocks(k, P.g.Vh, block, P.nrhs);
     const cudaError_t e = launch_k(hop64_kernel<E, D, MAT>, nb * P.nrhs, block, 0, s, P);
@@ -138,7 +147,7 @@ template <typename T, int R, int E, int D>
 cudaError_t run_hop(const HopParams& P, cudaStream_t s) {
     if constexpr (std::is_same<T, __half>::value) {
         if (P.arith16) {   // FP16 arithmetic (with or without a site-local block)
-            constexpr int blk = Hop16Bounds<R, D, false, 2>::THREADS;
+            const int blk = spread_block(P.g.Vh, P.nrhs, Hop16Bounds<R, D, false, 2>::THREADS);
             HopParams Q = P;
             Q.acc_exp = acc_exponent(P.a);
             constexpr int form = D == RED_NONE ? 0 : 1;
@@ -173,14 +182,14 @@ cudaError_t run_hop(const HopParams& P, cudaStream_t s) {
         if (P.fixed64) return P.mat ? run_hop64<E, D, true>(P, s) : run_hop64<E, D, false>(P, s);
     }
     if (P.mat) {   // with a site-local block (clover): the one-site-per-thread look-ahead kernel
-        const int blk = 128;
+        const int blk = spread_block(P.g.Vh, P.nrhs, 128);
         const void* km = (const void*)hop_kernel<T, R, E, D, true, false, true>;
         const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, blk) : reduce_blocks(km, P.g.Vh, blk, P.nrhs);
         { const cudaError_t le_ = launch_k(hop_kernel<T, R, E, D, true, false, true>, nb * P.nrhs, blk, 0, s, P); if (le_ != cudaSuccess) return le_; }
         return cudaGetLastError();
     }
     constexpr int form = D == RED_NONE ? 0 : 1;
-    const int block = P.block[form] > 0 ? P.block[form] : hop_block();
+    const int block = spread_block(P.g.Vh, P.nrhs, P.block[form] > 0 ? P.block[form] : hop_block());
     const int variant = P.variant[form] > 0 ? P.variant[form] : hop_variant();
     const int nr = P.nrhs;
     if constexpr (sizeof(T) == 2) {
@@ -297,14 +306,16 @@ cudaError_t Ops<T>::mat_from64(int n, const uint4* src64, uint4* dst, cudaStream
 template <typename T>
 cudaError_t Ops<T>::pupdate(int n, int nrhs, long long vs, uint4* p, const uint4* v, const uint4* r,
                             const SolverState* st, cudaStream_t s) {
-    { const cudaError_t le_ = launch_k(k_pupdate<T>, stream_blocks((n + Stream<T>::SITES - 1) / Stream<T>::SITES, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s, n, nrhs, vs, p, v, r, st); if (le_ != cudaSuccess) return le_; }
+    const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, VEC_BLOCK);
+    { const cudaError_t le_ = launch_k(k_pupdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, p, v, r, st); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::supdate(int n, int nrhs, long long vs, uint4* r, const uint4* v, const SolverState* st,
                             cudaStream_t s) {
-    { const cudaError_t le_ = launch_k(k_supdate<T>, stream_blocks((n + Stream<T>::SITES - 1) / Stream<T>::SITES, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s, n, nrhs, vs, r, v, st); if (le_ != cudaSuccess) return le_; }
+    const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, VEC_BLOCK);
+    { const cudaError_t le_ = launch_k(k_supdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, r, v, st); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
 
@@ -314,8 +325,8 @@ cudaError_t Ops<T>::xr(int mode, int n, int nrhs, long long vs, uint4* x, uint4*
                        SolverState* st, RedCtx rc, cudaStream_t s) {
 #define WD_XR_CASE(M)                                                                                        \
     if (mode == M) {                                                                                         \
-        const int nb = reduce_blocks((const void*)k_xr<T, M>, n, VEC_BLOCK, nrhs);                            \
-        { const cudaError_t le_ = launch_k(k_xr<T, M>, nb * nrhs, VEC_BLOCK, 0, s, n, nrhs, vs, x, r, p, t, rstar, xr_src, xp_src, st, rc); if (le_ != cudaSuccess) return le_; }   \
+        const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_xr<T, M>, n, block, nrhs);                            \
+        { const cudaError_t le_ = launch_k(k_xr<T, M>, nb * nrhs, block, 0, s, n, nrhs, vs, x, r, p, t, rstar, xr_src, xp_src, st, rc); if (le_ != cudaSuccess) return le_; }   \
         return cudaGetLastError();                                                                           \
     }
     WD_XR_CASE(XR_PLAIN)
@@ -328,39 +339,40 @@ cudaError_t Ops<T>::xr(int mode, int n, int nrhs, long long vs, uint4* x, uint4*
 template <typename T>
 cudaError_t Ops<T>::scale(int n, int nrhs, long long vs, uint4* r, uint4* x, const uint4* rstar, SolverState* st,
                           RedCtx rc, cudaStream_t s) {
-    const int nb = reduce_blocks((const void*)k_scale<T>, n, VEC_BLOCK, nrhs);
-    { const cudaError_t le_ = launch_k(k_scale<T>, nb * nrhs, VEC_BLOCK, 0, s, n, nrhs, vs, r, x, rstar, st, rc); if (le_ != cudaSuccess) return le_; }
+    const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_scale<T>, n, block, nrhs);
+    { const cudaError_t le_ = launch_k(k_scale<T>, nb * nrhs, block, 0, s, n, nrhs, vs, r, x, rstar, st, rc); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::rescale_in(int n, int nrhs, long long vs, long long vs64, const uint4* r64, uint4* r,
                                uint4* rstar, int ftz, SolverState* st, RedCtx rc, cudaStream_t s) {
-    const int nb = reduce_blocks((const void*)k_rescale_in<T>, n, VEC_BLOCK, nrhs);
-    k_rescale_in<T><<<nb * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, vs64, r64, r, rstar, ftz, st, rc);
+    const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_rescale_in<T>, n, block, nrhs);
+    k_rescale_in<T><<<nb * nrhs, block, 0, s>>>(n, nrhs, vs, vs64, r64, r, rstar, ftz, st, rc);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::correct(int n, int nrhs, long long vs, long long vs64, uint4* x64, const uint4* xt,
                             const SolverState* st, cudaStream_t s) {
-    k_correct<T><<<stream_blocks(n, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, vs64, x64, xt, st);
+    const int block = spread_block(n, nrhs, VEC_BLOCK);
+    k_correct<T><<<stream_blocks(n, block) * nrhs, block, 0, s>>>(n, nrhs, vs, vs64, x64, xt, st);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::norm2(int n, int nrhs, long long vs, const uint4* v, RedCtx rc, int guard_kind,
                           cudaStream_t s) {
-    const int nb = reduce_blocks((const void*)k_norm2<T>, n, VEC_BLOCK, nrhs);
-    k_norm2<T><<<nb * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, v, rc, guard_kind);
+    const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_norm2<T>, n, block, nrhs);
+    k_norm2<T><<<nb * nrhs, block, 0, s>>>(n, nrhs, vs, v, rc, guard_kind);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::odd_reconstruct(int n, int nrhs, long long vs, double kappa, const uint4* eta, const uint4* t,
                                     uint4* xo, RedCtx rc, cudaStream_t s) {
-    const int nb = reduce_blocks((const void*)k_odd_reconstruct<T>, n, VEC_BLOCK, nrhs);
-    k_odd_reconstruct<T><<<nb * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, kappa, eta, t, xo, rc);
+    const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_odd_reconstruct<T>, n, block, nrhs);
+    k_odd_reconstruct<T><<<nb * nrhs, block, 0, s>>>(n, nrhs, vs, kappa, eta, t, xo, rc);
     return cudaGetLastError();
 }
 
