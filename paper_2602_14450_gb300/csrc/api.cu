@@ -145,9 +145,11 @@ int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const ui
                         h->unit_dev, h->det_dev);
         const size_t bytes = (size_t)h->g.Vh * link_units(prec, recon) * 16;
         for (int p = 0; p < 2; ++p) {
-            uint4* buf = nullptr;
-            WD_CUDA(h, cudaMalloc(&buf, bytes));
-            h->links[prec][ri][p] = buf;
+            if (!h->link_buf[prec][ri][p]) {
+                WD_CUDA(h, cudaMalloc(&h->link_buf[prec][ri][p], bytes));
+                h->gen += 1;   // captured solver graphs hold the addresses
+            }
+            uint4* buf = h->link_buf[prec][ri][p];
             cudaError_t e = by_prec(prec, [&](auto tag) {
                 typedef typename decltype(tag)::type T;
                 return Ops<T>::build_links(recon, h->g, p, h->U64, buf, h->fixed64, 0);
@@ -155,6 +157,7 @@ int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const ui
             if (e != cudaSuccess) return cuda_fail(h, e, "build_links");
         }
         WD_CUDA(h, cudaDeviceSynchronize());
+        for (int p = 0; p < 2; ++p) h->links[prec][ri][p] = h->link_buf[prec][ri][p];
     }
     *even = h->links[prec][ri][0];
     *odd = h->links[prec][ri][1];
@@ -162,44 +165,68 @@ int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const ui
 }
 
 // max |U U^+ - 1| and max |det U - 1| over links, as bit patterns of
-// non-negative doubles (monotone as unsigned integers).
-__global__ void k_unitarity(int nlinks, const double* U, unsigned long long* out) {
-    double du = 0.0, dd = 0.0;
+// non-negative doubles (monotone as unsigned integers), and out[2] = 1 when an
+// element is NaN (which the maxima pass over). Bound by the FP64 pipe
+// (about 110 operations per link): the upper triangle of U U^+ only, and the
+// maxima are taken over squared moduli, with one square root per warp at the
+// end (a square root takes ~600 cycles; ten per link, and nine elements instead
+// of six, took 1526 us at 24^3 x 48; 487 us now).
+__global__ void __launch_bounds__(256) k_unitarity(int nlinks, const double* U, unsigned long long* out) {
+    unsigned long long mu = 0, md = 0;   // squared moduli as bit patterns
+    bool nan = false;
+    auto take = [&](unsigned long long& m, double re, double im) {
+        const unsigned long long q = (unsigned long long)__double_as_longlong(fma(im, im, re * re));
+        if (q > 0x7FF0000000000000ull) nan = true;
+        else if (q > m) m = q;
+    };
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += gridDim.x * blockDim.x) {
-        const double* m = U + (size_t)l * 18;
+        const double2* p = reinterpret_cast<const double2*>(U + (size_t)l * 18);
+        double m[18];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const double2 w = __ldg(p + e);
+            m[2 * e] = w.x;
+            m[2 * e + 1] = w.y;
+        }
+#pragma unroll
         for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) {
-                double re = 0, im = 0;
+#pragma unroll
+            for (int b = a; b < 3; ++b) {
+                double re = a == b ? -1.0 : 0.0, im = 0.0;
+#pragma unroll
                 for (int k = 0; k < 3; ++k) {   // sum_k U_ak conj(U_bk)
                     const double ar = m[2 * (3 * a + k)], ai = m[2 * (3 * a + k) + 1];
                     const double br = m[2 * (3 * b + k)], bi = m[2 * (3 * b + k) + 1];
-                    re += ar * br + ai * bi;
-                    im += ai * br - ar * bi;
+                    re = fma(ai, bi, fma(ar, br, re));
+                    if (a != b) im = fma(-ar, bi, fma(ai, br, im));
                 }
-                if (a == b) re -= 1.0;
-                du = fmax(du, sqrt(re * re + im * im));
+                take(mu, re, im);
             }
 #define R_(a, b) m[2 * (3 * (a) + (b))]
 #define I_(a, b) m[2 * (3 * (a) + (b)) + 1]
-        double dr = 0, di = 0;
+        double dr = -1.0, di = 0;
+#pragma unroll
         for (int b = 0; b < 3; ++b) {
             const int b1 = (b + 1) % 3, b2 = (b + 2) % 3;
-            const double cr = R_(1, b1) * R_(2, b2) - I_(1, b1) * I_(2, b2) - (R_(1, b2) * R_(2, b1) - I_(1, b2) * I_(2, b1));
-            const double ci = R_(1, b1) * I_(2, b2) + I_(1, b1) * R_(2, b2) - (R_(1, b2) * I_(2, b1) + I_(1, b2) * R_(2, b1));
-            dr += R_(0, b) * cr - I_(0, b) * ci;
-            di += R_(0, b) * ci + I_(0, b) * cr;
+            const double cr = fma(I_(1, b2), I_(2, b1), fma(-R_(1, b2), R_(2, b1), fma(-I_(1, b1), I_(2, b2), R_(1, b1) * R_(2, b2))));
+            const double ci = fma(-I_(1, b2), R_(2, b1), fma(-R_(1, b2), I_(2, b1), fma(I_(1, b1), R_(2, b2), R_(1, b1) * I_(2, b2))));
+            dr = fma(-I_(0, b), ci, fma(R_(0, b), cr, dr));
+            di = fma(I_(0, b), cr, fma(R_(0, b), ci, di));
         }
 #undef R_
 #undef I_
-        dd = fmax(dd, sqrt((dr - 1.0) * (dr - 1.0) + di * di));
+        take(md, dr, di);
     }
     for (int off = 16; off > 0; off >>= 1) {
-        du = fmax(du, __shfl_down_sync(0xffffffffu, du, off));
-        dd = fmax(dd, __shfl_down_sync(0xffffffffu, dd, off));
+        const unsigned long long a = __shfl_down_sync(0xffffffffu, mu, off), b = __shfl_down_sync(0xffffffffu, md, off);
+        mu = a > mu ? a : mu;
+        md = b > md ? b : md;
     }
+    const bool any = __any_sync(0xffffffffu, nan);
     if ((threadIdx.x & 31) == 0) {
-        atomicMax(out, (unsigned long long)__double_as_longlong(du));
-        atomicMax(out + 1, (unsigned long long)__double_as_longlong(dd));
+        atomicMax(out, (unsigned long long)__double_as_longlong(sqrt(__longlong_as_double((long long)mu))));
+        atomicMax(out + 1, (unsigned long long)__double_as_longlong(sqrt(__longlong_as_double((long long)md))));
+        if (any) atomicMax(out + 2, 1ull);
     }
 }
 
@@ -273,7 +300,7 @@ int wd_destroy(wd_handle* h) {
     for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 2; ++b)
             for (int c = 0; c < 2; ++c)
-                if (h->links[a][b][c]) cudaFree(h->links[a][b][c]);
+                if (h->link_buf[a][b][c]) cudaFree(h->link_buf[a][b][c]);
     if (h->U64) cudaFree(h->U64);
     if (h->st) cudaFree(h->st);
     if (h->partials) cudaFree(h->partials);
@@ -294,25 +321,24 @@ int wd_set_gauge(wd_handle* h, const double* U, int where) {
     if (!U || (where != WD_HOST && where != WD_DEVICE)) return fail(h, WD_ERR_INVALID_ARG, "bad gauge pointer or location");
     const size_t nl = (size_t)8 * h->g.Vh;   // 4 V links
     const size_t bytes = nl * 18 * sizeof(double);
+    // the links and clover blocks of the field before are rewritten in place: work on any stream that still reads
+    // them has to be done
+    if (h->have_gauge) WD_CUDA(h, cudaDeviceSynchronize());
     if (!h->U64) WD_CUDA(h, cudaMalloc(&h->U64, bytes));
     WD_CUDA(h, cudaMemcpy(h->U64, U, bytes, where == WD_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice));
     for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 2; ++b)
-            for (int c = 0; c < 2; ++c)
-                if (h->links[a][b][c]) {
-                    cudaFree(h->links[a][b][c]);
-                    h->links[a][b][c] = nullptr;
-                }
-    unsigned long long* dev = (unsigned long long*)workspace(h, "unitarity", 2 * sizeof(unsigned long long));
+            for (int c = 0; c < 2; ++c) h->links[a][b][c] = nullptr;
+    unsigned long long* dev = (unsigned long long*)workspace(h, "unitarity", 3 * sizeof(unsigned long long));
     if (!dev) return fail(h, WD_ERR_CUDA, "out of device memory");
-    WD_CUDA(h, cudaMemset(dev, 0, 2 * sizeof(unsigned long long)));
+    WD_CUDA(h, cudaMemset(dev, 0, 3 * sizeof(unsigned long long)));
     WD_CUDA(h, launch_unitarity((int)nl, h->U64, dev, 0));
-    unsigned long long host[2];
+    unsigned long long host[3];
     WD_CUDA(h, cudaMemcpy(host, dev, sizeof host, cudaMemcpyDeviceToHost));
     std::memcpy(&h->unit_dev, &host[0], sizeof(double));
     std::memcpy(&h->det_dev, &host[1], sizeof(double));
     // SU(3) links (the 12-real criterion) let the FP64 hop run in fixed point
-    const bool fixed64 = h->unit_dev <= SU3_DEV && h->det_dev <= SU3_DEV;
+    const bool fixed64 = h->unit_dev <= SU3_DEV && h->det_dev <= SU3_DEV && host[2] == 0;
     if (fixed64 != h->fixed64) {
         h->fixed64 = fixed64;
         h->gen += 1;   // captured solver graphs hold the other kernels
@@ -461,9 +487,9 @@ static int apply_n(wd_handle* h, int prec, int recon, int op, int nrhs, const vo
         if (cf_e) {   // out = C in first, then the hop adds to it in place
             e = by_prec(prec, [&](auto tag) {
                 typedef typename decltype(tag)::type T;
-                cudaError_t r2 = Ops<T>::apply_mat(h->g.Vh, nrhs, 2 * vsu, cf_e, (const uint4*)ie, (uint4*)oe, s);
+                cudaError_t r2 = Ops<T>::apply_chiral(h->g.Vh, nrhs, 2 * vsu, cf_e, (const uint4*)ie, (uint4*)oe, s);
                 if (r2 == cudaSuccess)
-                    r2 = Ops<T>::apply_mat(h->g.Vh, nrhs, 2 * vsu, cf_o, (const uint4*)(ie + half),
+                    r2 = Ops<T>::apply_chiral(h->g.Vh, nrhs, 2 * vsu, cf_o, (const uint4*)(ie + half),
                                            (uint4*)(oe + half), s);
                 return r2;
             });

@@ -473,43 +473,6 @@ __global__ void __launch_bounds__(256) k_rescale_in(int n, int nrhs, long long v
     grid_reduce<2, ST_INIT>(v, rc, sl);
 }
 
-// out = M in site by site (M: 12 x 12 complex blocks of one parity, shared by all right-hand sides)
-template <typename T>
-__global__ void __launch_bounds__(256) k_apply_mat(int n, int nrhs, long long vs, const uint4* mat, const uint4* in,
-                                                   uint4* out) {
-    typedef typename Unit<T>::C C;
-    const Slice sl = slice_of(nrhs);
-    in += sl.rhs * vs;
-    out += sl.rhs * vs;
-    RHS_LOOP(h, n) {
-        C v[24], o[24];
-        load_spinor<T>(in, n, h, v);
-        mat_mul<T>(mat, n, h, v, o);
-        store_spinor<T>(out, n, h, o);
-    }
-}
-
-// Blocks of storage T from FP64 blocks: 288 reals per site, element e of site h
-// in unit e / N of the block array (units n apart), as for spinors.
-template <typename T>
-__global__ void __launch_bounds__(256) k_mat_from64(int n, const uint4* src, uint4* dst) {
-    typedef typename Unit<T>::C C;
-    constexpr int N = Unit<T>::N;
-    GRID_STRIDE(h, n) {
-#pragma unroll 1
-        for (int u = 0; u < 288 / N; ++u) {
-            C v[N];
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                const int e = u * N + i;
-                const uint4 w = src[(size_t)(e / 2) * n + h];
-                v[i] = (C)Unit<double>::get(w, e % 2);
-            }
-            dst[(size_t)u * n + h] = Unit<T>::put(v);
-        }
-    }
-}
-
 // out = M in site by site with M in the chiral packing
 template <typename T>
 __global__ void __launch_bounds__(256) k_apply_chiral(int n, int nrhs, long long vs, const uint4* mat,
@@ -526,46 +489,19 @@ __global__ void __launch_bounds__(256) k_apply_chiral(int n, int nrhs, long long
     }
 }
 
-// Chiral packing of full FP64 blocks M (144 complex per site, element (i, j)
-// in unit 12 i + j): S_-/+ (k a, k' b) = (M[k a][k' b] -/+ M[k a][k'+2 b]
-// -/+ M[k+2 a][k' b] + M[k+2 a][k'+2 b]) / 4 with spin-colour index 3 s + a,
-// stored as described at mat_mul_chiral (block + first).
+// Blocks in the chiral packing (80 reals per site) of storage T from those in FP64.
 template <typename T>
-__global__ void __launch_bounds__(128) k_chiral_from64(int n, const uint4* src, uint4* dst) {
-    typedef typename Unit<T>::C C;
+__global__ void __launch_bounds__(256) k_chiral_from64(int n, const uint4* src, uint4* dst) {
     constexpr int N = Unit<T>::N;
+    const int u = blockIdx.y;
     GRID_STRIDE(h, n) {
-        for (int c = 0; c < 2; ++c) {
-            const double sg = c == 0 ? -1.0 : 1.0;
-            double blk[40];
-            for (int i = 0; i < 40; ++i) blk[i] = 0.0;
-            int q = 6;
-            for (int i = 0; i < 6; ++i)
-                for (int j = i; j < 6; ++j) {
-                    const int k = i / 3, a = i % 3, kk = j / 3, b = j % 3;
-                    const int r0 = 3 * k + a, r2 = 3 * (k + 2) + a, c0 = 3 * kk + b, c2 = 3 * (kk + 2) + b;
-                    double re = 0.0, im = 0.0;
-                    const int idx[4] = {12 * r0 + c0, 12 * r0 + c2, 12 * r2 + c0, 12 * r2 + c2};
-                    const double f[4] = {1.0, sg, sg, 1.0};
-                    for (int t = 0; t < 4; ++t) {
-                        const uint4 w = src[(size_t)idx[t] * n + h];
-                        re += f[t] * Unit<double>::get(w, 0);
-                        im += f[t] * Unit<double>::get(w, 1);
-                    }
-                    if (i == j) {
-                        blk[i] = 0.25 * re;
-                    } else {
-                        blk[q] = 0.25 * re;
-                        blk[q + 1] = 0.25 * im;
-                        q += 2;
-                    }
-                }
-            for (int u = 0; u < 40 / N; ++u) {
-                C v[N];
-                for (int e = 0; e < N; ++e) v[e] = (C)blk[u * N + e];
-                dst[(size_t)(c * (40 / N) + u) * n + h] = Unit<T>::put(v);
-            }
+        alignas(16) T v[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int e = u * N + i;
+            v[i] = from_double<T>(Unit<double>::get(__ldg(src + (size_t)(e / 2) * n + h), e % 2));
         }
+        dst[(size_t)u * n + h] = *reinterpret_cast<const uint4*>(v);
     }
 }
 
@@ -666,48 +602,58 @@ __global__ void k_unpack(Geom g, int parity, const uint4* in, double* lex) {
 }
 
 // Gathered links of output parity p (see hop_impl.cuh) from FP64 lex links.
-// FIXED: every FP64 real as its two fixed-point digits (fixed64.cuh).
+// FIXED: every FP64 real as its two fixed-point digits (fixed64.cuh). A thread
+// takes one site and the smallest group of links that fills whole 16-byte
+// units (blockIdx.y), reads each link as nine 16-byte words and writes units.
+// Bound by memory: 70 us (FP16, 12-real) and 221 us (FP64, 18-real) per parity
+// at 24^3 x 48; one thread per site writing real by real took 268 and 241 us.
+template <typename T, int R> struct LinkGroup {
+    static constexpr int B = R * (int)sizeof(T);
+    static constexpr int G = B % 16 == 0 ? 1 : (2 * B) % 16 == 0 ? 2 : 4;
+};
 template <typename T, int R, bool FIXED>
-__global__ void k_build_links(Geom g, int parity, const double* U, uint4* out) {
-    constexpr int N = Unit<T>::N;
-    const int V = 2 * g.Vh;
+__global__ void __launch_bounds__(256) k_build_links(Geom g, int parity, const double* U, uint4* out) {
+    constexpr int N = Unit<T>::N, G = LinkGroup<T, R>::G;
+    const size_t V = 2 * (size_t)g.Vh;
     GRID_STRIDE(h, g.Vh) {
-        const int s = lex_of(g, parity, h);
-        int c[4];
-        c[0] = s % g.L[0];
-        c[1] = (s / g.L[0]) % g.L[1];
-        c[2] = (s / (g.L[0] * g.L[1])) % g.L[2];
-        c[3] = s / (g.L[0] * g.L[1] * g.L[2]);
-        for (int mu = 0; mu < 4; ++mu) {
-            int cm[4] = {c[0], c[1], c[2], c[3]};
-            cm[mu] = (c[mu] + g.L[mu] - 1) % g.L[mu];
-            const int sm = cm[0] + g.L[0] * (cm[1] + g.L[1] * (cm[2] + g.L[2] * cm[3]));
-            const double* uf = U + ((size_t)mu * V + s) * 18;
-            const double* ub = U + ((size_t)mu * V + sm) * 18;
+        const Coord c = coord_of(g, parity, h);
+        const int s = c.x + g.L[0] * c.row;
+        alignas(16) T v[G * R];
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            const int d = blockIdx.y * G + j, mu = d >> 1;
+            const bool back = d & 1;
+            bool wrap;
+            const int hn = neighbour(g, h, c, d, &wrap);   // the site a hop in direction d comes from
+            const int site = back ? lex_of(g, 1 - parity, hn) : s;
+            const double2* p = reinterpret_cast<const double2*>(U + ((size_t)mu * V + site) * 18);
+            double m[18];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                const double2 w = __ldg(p + e);
+                m[2 * e] = w.x;
+                m[2 * e + 1] = w.y;
+            }
             // a direction split across processes: the hops that leave the sub-lattice are
             // remote, and their links are stored as zeros (the face terms are added apart)
-            const bool split = (g.part >> mu) & 1u;
-            const bool zf = split && c[mu] == g.L[mu] - 1, zb = split && c[mu] == 0;
+            const bool zero = wrap && ((g.part >> mu) & 1u);
+#pragma unroll
             for (int e = 0; e < R; ++e) {
                 // forward: U_mu(x)[a][b]; backward: (U_mu(x-mu)^+)[a][b] = conj(U_mu(x-mu)[b][a])
-                const int a = e / 6, b = (e % 6) / 2, im = e & 1;
-                const double vf = zf ? 0.0 : uf[e];
-                const double vb = zb ? 0.0 : (im ? -ub[2 * (3 * b + a) + 1] : ub[2 * (3 * b + a)]);
-                const int ef = (2 * mu) * R + e, eb = (2 * mu + 1) * R + e;
-                T* const of = reinterpret_cast<T*>(out + (size_t)(ef / N) * g.Vh + h) + ef % N;
-                T* const ob = reinterpret_cast<T*>(out + (size_t)(eb / N) * g.Vh + h) + eb % N;
+                const int a = e / 6, b = (e % 6) / 2, im = e & 1, t = 2 * (3 * b + a) + im;
+                const double x = zero ? 0.0 : back ? (im ? -m[t] : m[t]) : m[e];
                 if constexpr (FIXED) {
-                    int2 wf, wb;
-                    fx::link_digits(vf, wf.x, wf.y);
-                    fx::link_digits(vb, wb.x, wb.y);
-                    *reinterpret_cast<int2*>(of) = wf;
-                    *reinterpret_cast<int2*>(ob) = wb;
+                    int lo, hi;
+                    fx::link_digits(x, lo, hi);
+                    v[j * R + e] = __hiloint2double(hi, lo);
                 } else {
-                    *of = from_double<T>(vf);
-                    *ob = from_double<T>(vb);
+                    v[j * R + e] = from_double<T>(x);
                 }
             }
         }
+#pragma unroll
+        for (int u = 0; u < G * R / N; ++u)
+            out[(size_t)(blockIdx.y * (G * R / N) + u) * g.Vh + h] = *reinterpret_cast<const uint4*>(&v[u * N]);
     }
 }
 

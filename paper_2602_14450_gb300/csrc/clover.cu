@@ -4,198 +4,404 @@
 //   sigma_mu_nu = (i/2) [gamma_mu, gamma_nu],
 //   Fh_mu_nu = traceless part of (Q_mu_nu - Q_mu_nu^+) / (8 i),
 // Q_mu_nu(x) the four plaquettes of the mu-nu plane with a corner at x, each
-// traversed mu-then-nu. Built once per gauge field in FP64, one thread per
-// site: C and C^{-1} (Gauss-Jordan with partial pivoting) are written as
-// 12 x 12 complex blocks (row-major, spin-colour index 3 s + a) per parity in
-// the unit layout of the spinors. The operators use C^-1 in the chiral packing
-// (two Hermitian 6 x 6 blocks, 80 reals per site; see mat_mul_chiral), made
-// on first use per precision; C itself (full) serves the true residual.
+// traversed mu-then-nu. Built once per gauge field; C and C^-1 are stored in
+// FP64 in the chiral packing (two Hermitian 6 x 6 blocks, 80 reals per site;
+// see mat_mul_chiral), other precisions are made from it on first use.
+//
+// In the chiral combinations the spin matrices are Pauli matrices:
+// sigma_ij = -eps_ijk sigma_k and sigma_k4 = -(off-diagonal) sigma_k, so block
+// c (sg = -1, +1) is
+//   S = 1/2 + (c_sw kappa / 2) sum_k sigma_k (x) G_k,   G = (F_12 + sg F_03, -F_02 + sg F_13, F_01 + sg F_23)
+// (directions 0..3 = x, y, z, t), and the packing of C^-1 is S^-1 / 4.
 #include <algorithm>
 #include <cmath>
 #include <string>
+#include <type_traits>
 
+#include "fixed64.cuh"
 #include "handle.h"
 
 namespace wd {
 
 namespace {
 
-struct Z {
-    double r, i;
-};
-__device__ __forceinline__ Z zmul(Z a, Z b) { return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r}; }
-__device__ __forceinline__ Z zadd(Z a, Z b) { return {a.r + b.r, a.i + b.i}; }
-__device__ __forceinline__ Z zsub(Z a, Z b) { return {a.r - b.r, a.i - b.i}; }
-__device__ __forceinline__ Z zconj(Z a) { return {a.r, -a.i}; }
-
-struct M3 {
-    Z e[3][3];
+template <typename R> struct Vec3 {
+    R v[6];   // three complex numbers
 };
 
-__device__ M3 mul(const M3& a, const M3& b) {
-    M3 c;
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            Z s = {0, 0};
-            for (int k = 0; k < 3; ++k) s = zadd(s, zmul(a.e[i][k], b.e[k][j]));
-            c.e[i][j] = s;
-        }
-    return c;
-}
+// The links of a site as matrices of the products below. FIXED: the gathered
+// FP64 links as fixed-point digits (SU(3) links), vectors 64-bit integers in
+// units of 2^-59 (fixed64.cuh; the products' magnitudes stay at or below 2);
+// otherwise the FP64 links in the host layout and FP64 arithmetic.
+struct Field {
+    const double* U;
+    const uint4* l[2];
+    long long V;
+    int Vh;
+};
+struct Site {
+    int lex, p;   // lexicographic index and parity
+};
 
-__device__ M3 dag(const M3& a) {
-    M3 c;
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) c.e[i][j] = zconj(a.e[j][i]);
-    return c;
-}
+template <bool FIXED> struct Links;
 
-// Lexicographic index of the site at coordinates c shifted by (s0 mu-hat + s1 nu-hat), periodic.
-__device__ long long shifted(const Geom& g, const int (&c)[4], int mu, int s0, int nu, int s1) {
-    int d[4] = {c[0], c[1], c[2], c[3]};
-    d[mu] = (d[mu] + s0 + g.L[mu]) % g.L[mu];
-    d[nu] = (d[nu] + s1 + g.L[nu]) % g.L[nu];
-    return d[0] + (long long)g.L[0] * (d[1] + (long long)g.L[1] * (d[2] + (long long)g.L[2] * d[3]));
-}
-
-__device__ M3 link(const double* U, long long V, int mu, long long site) {
-    const double* p = U + ((size_t)mu * V + site) * 18;
-    M3 m;
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) m.e[a][b] = {p[2 * (3 * a + b)], p[2 * (3 * a + b) + 1]};
-    return m;
-}
-
-// gamma_mu[s][t] in the Dirac representation: gamma_k = [[0, -i sigma_k], [i sigma_k, 0]], gamma_4 = diag(1, 1, -1, -1).
-__device__ Z gamma_el(int mu, int s, int t) {
-    if (mu == 3) return {(s == t) ? (s < 2 ? 1.0 : -1.0) : 0.0, 0.0};
-    const bool upper = s < 2, tupper = t < 2;
-    if (upper == tupper) return {0, 0};
-    const int a = s & 1, b = t & 1;
-    Z p;   // Pauli sigma_{mu+1}[a][b]
-    if (mu == 0) p = {(a != b) ? 1.0 : 0.0, 0.0};
-    else if (mu == 1) p = (a == b) ? Z{0, 0} : (a == 0 ? Z{0, -1} : Z{0, 1});
-    else p = (a != b) ? Z{0, 0} : Z{a == 0 ? 1.0 : -1.0, 0.0};
-    const Z f = upper ? Z{0, -1} : Z{0, 1};   // -i (upper right block) or +i (lower left block)
-    return zmul(f, p);
-}
-
-// sigma_mu_nu[s][t] = (i/2) sum_u (gamma_mu[s][u] gamma_nu[u][t] - gamma_nu[s][u] gamma_mu[u][t])
-__device__ Z sigma_el(int mu, int nu, int s, int t) {
-    Z c = {0, 0};
-    for (int u = 0; u < 4; ++u)
-        c = zadd(c, zsub(zmul(gamma_el(mu, s, u), gamma_el(nu, u, t)), zmul(gamma_el(nu, s, u), gamma_el(mu, u, t))));
-    return zmul(Z{0, 0.5}, c);
-}
-
-__device__ void store_block(uint4* dst, int Vh, int h, const Z (&m)[12][12]) {
-    for (int i = 0; i < 12; ++i)
-        for (int j = 0; j < 12; ++j) {
-            uint4 w;
-            w.x = (unsigned)__double2loint(m[i][j].r);
-            w.y = (unsigned)__double2hiint(m[i][j].r);
-            w.z = (unsigned)__double2loint(m[i][j].i);
-            w.w = (unsigned)__double2hiint(m[i][j].i);
-            dst[(size_t)(12 * i + j) * Vh + h] = w;
-        }
-}
-
-__global__ void __launch_bounds__(128) k_clover_build(Geom g, const double* U, double ck, uint4* fwd_e, uint4* fwd_o,
-                                                      uint4* inv_e, uint4* inv_o, int* singular) {
-    const long long V = 2LL * g.Vh;
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < V; s += (long long)gridDim.x * blockDim.x) {
-        int c[4];
-        long long r = s;
-        c[0] = (int)(r % g.L[0]); r /= g.L[0];
-        c[1] = (int)(r % g.L[1]); r /= g.L[1];
-        c[2] = (int)(r % g.L[2]); r /= g.L[2];
-        c[3] = (int)r;
-        const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
-        const int h = (int)(s / 2);
-        Z a[12][12];
-        for (int i = 0; i < 12; ++i)
-            for (int j = 0; j < 12; ++j) a[i][j] = {i == j ? 1.0 : 0.0, 0.0};
-        for (int mu = 0; mu < 4; ++mu)
-            for (int nu = mu + 1; nu < 4; ++nu) {
-                const M3 um = link(U, V, mu, s), un = link(U, V, nu, s);
-                M3 q = mul(mul(mul(um, link(U, V, nu, shifted(g, c, mu, 1, nu, 0))),
-                               dag(link(U, V, mu, shifted(g, c, mu, 0, nu, 1)))),
-                           dag(un));
-                M3 l = mul(mul(mul(un, dag(link(U, V, mu, shifted(g, c, mu, -1, nu, 1)))),
-                               dag(link(U, V, nu, shifted(g, c, mu, -1, nu, 0)))),
-                           link(U, V, mu, shifted(g, c, mu, -1, nu, 0)));
-                for (int i = 0; i < 3; ++i)
-                    for (int j = 0; j < 3; ++j) q.e[i][j] = zadd(q.e[i][j], l.e[i][j]);
-                l = mul(mul(mul(dag(link(U, V, mu, shifted(g, c, mu, -1, nu, 0))),
-                                dag(link(U, V, nu, shifted(g, c, mu, -1, nu, -1)))),
-                            link(U, V, mu, shifted(g, c, mu, -1, nu, -1))),
-                        link(U, V, nu, shifted(g, c, mu, 0, nu, -1)));
-                for (int i = 0; i < 3; ++i)
-                    for (int j = 0; j < 3; ++j) q.e[i][j] = zadd(q.e[i][j], l.e[i][j]);
-                l = mul(mul(mul(dag(link(U, V, nu, shifted(g, c, mu, 0, nu, -1))),
-                                link(U, V, mu, shifted(g, c, mu, 0, nu, -1))),
-                            link(U, V, nu, shifted(g, c, mu, 1, nu, -1))),
-                        dag(um));
-                for (int i = 0; i < 3; ++i)
-                    for (int j = 0; j < 3; ++j) q.e[i][j] = zadd(q.e[i][j], l.e[i][j]);
-                // F = (Q - Q^+) / (8 i), then its traceless part
-                Z f[3][3];
-                for (int i = 0; i < 3; ++i)
-                    for (int j = 0; j < 3; ++j) {
-                        const Z d = zsub(q.e[i][j], zconj(q.e[j][i]));
-                        f[i][j] = {d.i / 8.0, -d.r / 8.0};   // d / (8 i)
-                    }
-                const Z tr = {(f[0][0].r + f[1][1].r + f[2][2].r) / 3.0, (f[0][0].i + f[1][1].i + f[2][2].i) / 3.0};
-                for (int i = 0; i < 3; ++i) f[i][i] = zsub(f[i][i], tr);
-                for (int s1 = 0; s1 < 4; ++s1)
-                    for (int t1 = 0; t1 < 4; ++t1) {
-                        const Z sg = sigma_el(mu, nu, s1, t1);
-                        if (sg.r == 0.0 && sg.i == 0.0) continue;
-                        for (int i = 0; i < 3; ++i)
-                            for (int j = 0; j < 3; ++j) {
-                                const Z v = zmul(sg, f[i][j]);
-                                a[3 * s1 + i][3 * t1 + j] = zsub(a[3 * s1 + i][3 * t1 + j], Z{ck * v.r, ck * v.i});
-                            }
-                    }
-            }
-        store_block(p == 0 ? fwd_e : fwd_o, g.Vh, h, a);
-        // inverse by Gauss-Jordan elimination with partial pivoting
-        Z inv[12][12];
-        for (int i = 0; i < 12; ++i)
-            for (int j = 0; j < 12; ++j) inv[i][j] = {i == j ? 1.0 : 0.0, 0.0};
-        bool ok = true;
-        for (int col = 0; col < 12; ++col) {
-            int piv = col;
-            double best = -1.0;
-            for (int i = col; i < 12; ++i) {
-                const double m = a[i][col].r * a[i][col].r + a[i][col].i * a[i][col].i;
-                if (m > best) { best = m; piv = i; }
-            }
-            if (!(best > 0.0)) { ok = false; break; }
-            if (piv != col)
-                for (int j = 0; j < 12; ++j) {
-                    Z t = a[col][j]; a[col][j] = a[piv][j]; a[piv][j] = t;
-                    t = inv[col][j]; inv[col][j] = inv[piv][j]; inv[piv][j] = t;
-                }
-            const Z d = a[col][col];
-            const Z rd = {d.r / best, -d.i / best};   // 1 / d
-            for (int j = 0; j < 12; ++j) {
-                a[col][j] = zmul(a[col][j], rd);
-                inv[col][j] = zmul(inv[col][j], rd);
-            }
-            for (int i = 0; i < 12; ++i) {
-                if (i == col) continue;
-                const Z fct = a[i][col];
-                if (fct.r == 0.0 && fct.i == 0.0) continue;
-                for (int j = 0; j < 12; ++j) {
-                    a[i][j] = zsub(a[i][j], zmul(fct, a[col][j]));
-                    inv[i][j] = zsub(inv[i][j], zmul(fct, inv[col][j]));
-                }
-            }
-        }
-        if (!ok) atomicExch(singular, 1);
-        store_block(p == 0 ? inv_e : inv_o, g.Vh, h, inv);
+template <> struct Links<true> {
+    typedef long long R;
+    static __device__ __forceinline__ const uint4* at(const Field& f, Site s, int mu) {
+        return (s.p ? f.l[1] : f.l[0]) + (size_t)(18 * mu) * f.Vh + (s.lex >> 1);
     }
+    // entry i of column j of the matrix: U, its transpose (T), complex conjugate (C) or both
+    template <bool T, bool C>
+    static __device__ __forceinline__ Vec3<R> column(const Field& f, Site s, int mu, int j) {
+        const uint4* m = at(f, s, mu);
+        Vec3<R> o;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const uint4 w = __ldg(m + (size_t)(T ? 3 * j + i : 3 * i + j) * f.Vh);
+            const R re = ((R)(int)w.y << 32) + (int)w.x, im = ((R)(int)w.w << 32) + (int)w.z;
+            o.v[2 * i] = re >> 2;
+            o.v[2 * i + 1] = C ? -(im >> 2) : im >> 2;
+        }
+        return o;
+    }
+    template <bool T, bool C>
+    static __device__ __noinline__ Vec3<R> mul(const uint4* m, int Vh, Vec3<R> v) {
+        int h0[6], h1[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) fx::digits(v.v[i], h0[i], h1[i]);
+        Vec3<R> o;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            int u0[6], u1[6], n0[3], n1[3];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const uint4 w = __ldg(m + (size_t)(T ? 3 * j + i : 3 * i + j) * Vh);
+                u0[2 * j] = (int)w.x;
+                u1[2 * j] = (int)w.y;
+                u0[2 * j + 1] = C ? -(int)w.z : (int)w.z;
+                u1[2 * j + 1] = C ? -(int)w.w : (int)w.w;
+                n0[j] = C ? (int)w.z : -(int)w.z;
+                n1[j] = C ? (int)w.w : -(int)w.w;
+            }
+            long long re, im;
+            fx::row_mul(u0, u1, n0, n1, h0, h1, re, im);
+            o.v[2 * i] = re * 8;
+            o.v[2 * i + 1] = im * 8;
+        }
+        return o;
+    }
+    template <bool T, bool C>
+    static __device__ __forceinline__ Vec3<R> mul(const Field& f, Site s, int mu, Vec3<R> v) {
+        return mul<T, C>(at(f, s, mu), f.Vh, v);
+    }
+    static __device__ __forceinline__ double real(R v) { return (double)v * (1.0 / 576460752303423488.0); }   // 2^-59
+};
+
+template <> struct Links<false> {
+    typedef double R;
+    static __device__ __forceinline__ const double* at(const Field& f, Site s, int mu) {
+        return f.U + ((size_t)mu * f.V + s.lex) * 18;
+    }
+    template <bool T, bool C>
+    static __device__ __forceinline__ Vec3<R> column(const Field& f, Site s, int mu, int j) {
+        const double* m = at(f, s, mu);
+        Vec3<R> o;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int e = 2 * (T ? 3 * j + i : 3 * i + j);
+            o.v[2 * i] = m[e];
+            o.v[2 * i + 1] = C ? -m[e + 1] : m[e + 1];
+        }
+        return o;
+    }
+    template <bool T, bool C>
+    static __device__ __noinline__ Vec3<R> mul(const double* m, Vec3<R> v) {
+        Vec3<R> o;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            double re = 0.0, im = 0.0;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int e = 2 * (T ? 3 * j + i : 3 * i + j);
+                const double a = m[e], b = C ? -m[e + 1] : m[e + 1];
+                re = fma(-b, v.v[2 * j + 1], fma(a, v.v[2 * j], re));
+                im = fma(b, v.v[2 * j], fma(a, v.v[2 * j + 1], im));
+            }
+            o.v[2 * i] = re;
+            o.v[2 * i + 1] = im;
+        }
+        return o;
+    }
+    template <bool T, bool C>
+    static __device__ __forceinline__ Vec3<R> mul(const Field& f, Site s, int mu, Vec3<R> v) {
+        return mul<T, C>(at(f, s, mu), v);
+    }
+    static __device__ __forceinline__ double real(R v) { return v; }
+};
+
+// Site at coordinates c shifted by a mu-hat + b nu-hat (a, b in -1..1), periodic.
+__device__ __forceinline__ Site shifted(const Geom& g, const Coord& c, int mu, int a, int nu, int b) {
+    int d[4] = {c.x, c.y, c.z, c.t};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int s = (i == mu ? a : 0) + (i == nu ? b : 0);
+        d[i] += s;
+        if (d[i] < 0) d[i] += g.L[i];
+        if (d[i] >= g.L[i]) d[i] -= g.L[i];
+    }
+    return {d[0] + g.L[0] * (d[1] + g.L[1] * (d[2] + g.L[2] * d[3])), (d[0] + d[1] + d[2] + d[3]) & 1};
+}
+
+// Q - Q^+ of plane (mu, nu) from two products of three links each. The leaves L1..L4 enter only through their
+// anti-Hermitian parts, so L2 may be replaced by -L2^+, which ends with U_nu(x)^+ as L1 does, and L4 by -L4^+,
+// which ends with U_nu(x - nu) as L3 does:
+//   L1 - L2^+ = [U_mu(x) U_nu(x+mu) U_mu(x+nu)^+ - U_mu(x-mu)^+ U_nu(x-mu) U_mu(x-mu+nu)] U_nu(x)^+
+//   L3 - L4^+ = [U_mu(x-mu)^+ U_nu(x-mu-nu)^+ U_mu(x-mu-nu) - U_mu(x) U_nu(x+mu-nu)^+ U_mu(x-nu)^+] U_nu(x-nu)
+// (10 matrix products instead of 12). Writes the 9 reals of F before the trace is taken out: diagonal, then the
+// complex elements (0,1), (0,2), (1,2).
+template <bool FIXED>
+__device__ void plane_field(const Geom& g, const Field& f, const Coord& c, int mu, int nu, double (&F)[9]) {
+    typedef Links<FIXED> L;
+    typedef typename L::R R;
+    const Site x = shifted(g, c, mu, 0, nu, 0), xm = shifted(g, c, mu, -1, nu, 0), xn = shifted(g, c, mu, 0, nu, -1);
+    R q[3][6];
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        Vec3<R> X[3];   // columns
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            Vec3<R> a, b;
+            if (half == 0) {
+                const Site pn = shifted(g, c, mu, 0, nu, 1), pm = shifted(g, c, mu, 1, nu, 0);
+                const Site mp = shifted(g, c, mu, -1, nu, 1);
+                a = L::template column<true, true>(f, pn, mu, j);
+                a = L::template mul<false, false>(f, pm, nu, a);
+                a = L::template mul<false, false>(f, x, mu, a);
+                b = L::template column<false, false>(f, mp, mu, j);
+                b = L::template mul<false, false>(f, xm, nu, b);
+                b = L::template mul<true, true>(f, xm, mu, b);
+            } else {
+                const Site mm = shifted(g, c, mu, -1, nu, -1), pm = shifted(g, c, mu, 1, nu, -1);
+                a = L::template column<false, false>(f, mm, mu, j);
+                a = L::template mul<true, true>(f, mm, nu, a);
+                a = L::template mul<true, true>(f, xm, mu, a);
+                b = L::template column<true, true>(f, xn, mu, j);
+                b = L::template mul<true, true>(f, pm, nu, b);
+                b = L::template mul<false, false>(f, x, mu, b);
+            }
+#pragma unroll
+            for (int e = 0; e < 6; ++e) X[j].v[e] = a.v[e] - b.v[e];
+        }
+        // row i of X W: the vector X_i. through W^T
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            Vec3<R> r;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                r.v[2 * j] = X[j].v[2 * i];
+                r.v[2 * j + 1] = X[j].v[2 * i + 1];
+            }
+            r = half == 0 ? L::template mul<false, true>(f, x, nu, r) : L::template mul<true, false>(f, xn, nu, r);
+#pragma unroll
+            for (int e = 0; e < 6; ++e) q[i][e] = half == 0 ? r.v[e] : q[i][e] + r.v[e];
+        }
+    }
+    // F = (Q - Q^+) / (8 i): (re, im) -> (im, -re) / 8
+#pragma unroll
+    for (int i = 0; i < 3; ++i) F[i] = 0.25 * L::real(q[i][2 * i + 1]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int i = k < 2 ? 0 : 1, j = k < 1 ? 1 : 2;
+        F[3 + 2 * k] = 0.125 * L::real(q[i][2 * j + 1] + q[j][2 * i + 1]);
+        F[4 + 2 * k] = -0.125 * L::real(q[i][2 * j] - q[j][2 * i]);
+    }
+}
+
+// Inverse of a Hermitian 6 x 6 block by Gauss-Jordan with partial pivoting; false when a pivot vanishes. For
+// the blocks whose plain pivots are small (a strongly indefinite block).
+__device__ __noinline__ bool invert_pivoted(const double* S, double* out) {
+    double a[6][12], inv[6][12];
+    for (int i = 0; i < 6; ++i)
+        for (int j = 0; j < 6; ++j) {
+            const int lo = i < j ? i : j, hi = i < j ? j : i;
+            const int q = 6 + 2 * (lo * 5 - lo * (lo - 1) / 2 + hi - lo - 1);
+            a[i][2 * j] = i == j ? S[i] : S[q];
+            a[i][2 * j + 1] = i == j ? 0.0 : i < j ? S[q + 1] : -S[q + 1];
+            inv[i][2 * j] = i == j ? 1.0 : 0.0;
+            inv[i][2 * j + 1] = 0.0;
+        }
+    for (int col = 0; col < 6; ++col) {
+        int piv = col;
+        double best = -1.0;
+        for (int i = col; i < 6; ++i) {
+            const double m = a[i][2 * col] * a[i][2 * col] + a[i][2 * col + 1] * a[i][2 * col + 1];
+            if (m > best) { best = m; piv = i; }
+        }
+        if (!(best > 0.0)) return false;
+        for (int j = 0; j < 12 && piv != col; ++j) {
+            double t = a[col][j]; a[col][j] = a[piv][j]; a[piv][j] = t;
+            t = inv[col][j]; inv[col][j] = inv[piv][j]; inv[piv][j] = t;
+        }
+        const double dr = a[col][2 * col] / best, di = -a[col][2 * col + 1] / best;   // 1 / pivot
+        for (int j = 0; j < 6; ++j) {
+            double r = a[col][2 * j], i = a[col][2 * j + 1];
+            a[col][2 * j] = r * dr - i * di;
+            a[col][2 * j + 1] = r * di + i * dr;
+            r = inv[col][2 * j];
+            i = inv[col][2 * j + 1];
+            inv[col][2 * j] = r * dr - i * di;
+            inv[col][2 * j + 1] = r * di + i * dr;
+        }
+        for (int i = 0; i < 6; ++i) {
+            if (i == col) continue;
+            const double fr = a[i][2 * col], fi = a[i][2 * col + 1];
+            for (int j = 0; j < 6; ++j) {
+                a[i][2 * j] -= fr * a[col][2 * j] - fi * a[col][2 * j + 1];
+                a[i][2 * j + 1] -= fr * a[col][2 * j + 1] + fi * a[col][2 * j];
+                inv[i][2 * j] -= fr * inv[col][2 * j] - fi * inv[col][2 * j + 1];
+                inv[i][2 * j + 1] -= fr * inv[col][2 * j + 1] + fi * inv[col][2 * j];
+            }
+        }
+    }
+    for (int i = 0, q = 6; i < 6; ++i) {
+        out[i] = inv[i][2 * i];
+        for (int j = i + 1; j < 6; ++j, q += 2) {
+            out[q] = inv[i][2 * j];
+            out[q + 1] = inv[i][2 * j + 1];
+        }
+    }
+    return true;
+}
+
+// Element (i, j), i != j, of a Hermitian matrix stored as 6 reals and the upper triangle (row by row).
+__host__ __device__ constexpr int tri(int i, int j) { return 6 + 2 * (i * 5 - i * (i - 1) / 2 + j - i - 1); }
+__device__ __forceinline__ void element(const double (&s)[36], int i, int j, double& re, double& im) {
+    re = s[i < j ? tri(i, j) : tri(j, i)];
+    im = i < j ? s[tri(i, j) + 1] : -s[tri(j, i) + 1];
+}
+
+// s := s^-1 for a Hermitian 6 x 6 block by the sweep operator (each sweep keeps the matrix Hermitian, so only the
+// triangle is held; after all six it is -s^-1). Pivots are not exchanged; false when one is below 1e-3 of the
+// block's scale 1/2 (the trace of the block is 3).
+__device__ __forceinline__ bool sweep_inverse(double (&s)[36]) {
+    bool good = true;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        good = good && fabs(s[k]) > 5e-4;
+        const double rd = 1.0 / s[k];
+        double cr[6], ci[6];   // column k
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+            if (i != k) element(s, i, k, cr[i], ci[i]);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            if (i == k) continue;
+            const double br = cr[i] * rd, bi = ci[i] * rd;   // s_ik / s_kk
+            s[i] = fma(-br, cr[i], fma(-bi, ci[i], s[i]));
+#pragma unroll
+            for (int j = i + 1; j < 6; ++j) {
+                if (j == k) continue;                        // s_ij -= s_ik conj(s_jk) / s_kk
+                s[tri(i, j)] = fma(-br, cr[j], fma(-bi, ci[j], s[tri(i, j)]));
+                s[tri(i, j) + 1] = fma(-bi, cr[j], fma(br, ci[j], s[tri(i, j) + 1]));
+            }
+            if (i < k) {
+                s[tri(i, k)] = br;
+                s[tri(i, k) + 1] = bi;
+            } else {
+                s[tri(k, i)] = br;
+                s[tri(k, i) + 1] = -bi;
+            }
+        }
+        s[k] = -rd;
+    }
+#pragma unroll
+    for (int i = 0; i < 36; ++i) s[i] = -s[i];
+    return good;
+}
+
+// Packed block c of site h: 36 reals and 4 zeros as 20 units.
+__device__ __forceinline__ void store_chiral(uint4* dst, int Vh, int h, int c, const double (&s)[36]) {
+#pragma unroll
+    for (int u = 0; u < 20; ++u) {
+        const double v[2] = {u < 18 ? s[2 * u < 36 ? 2 * u : 0] : 0.0, u < 18 ? s[2 * u + 1 < 36 ? 2 * u + 1 : 0] : 0.0};
+        dst[(size_t)(20 * c + u) * Vh + h] = Unit<double>::put(v);
+    }
+}
+
+// One block takes 32 sites of one parity (blockIdx.y): each of its six warps
+// forms the field strength of one plane, then warps 0 and 1 assemble and
+// invert one chiral block each. Bound: in FP64 arithmetic the products (6480
+// multiply-adds per site) keep the FP64 pipe busy; in fixed point they take the
+// integer multiplier a quarter of that time, and the inverses (~1000 FP64
+// operations) are half of the rest. Measured at 24^3 x 48: 3.3 ms, against
+// 53.7 ms with one thread per site and 12 x 12 blocks in local memory.
+template <bool FIXED>
+__global__ void __launch_bounds__(192) k_clover_build(Geom g, Field f, double ck, uint4* fwd_e, uint4* fwd_o,
+                                                      uint4* inv_e, uint4* inv_o, int* singular) {
+    __shared__ double F[6][9][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = blockIdx.y;
+    const int h = blockIdx.x * 32 + lane;
+    const bool ok = h < g.Vh;
+    if (ok) {
+        const int mu = warp < 3 ? 0 : warp < 5 ? 1 : 2;
+        const int nu = warp < 3 ? warp + 1 : warp < 5 ? warp - 1 : 3;
+        double t[9];
+        plane_field<FIXED>(g, f, coord_of(g, p, h), mu, nu, t);
+        const double tr = (t[0] + t[1] + t[2]) / 3.0;
+        for (int i = 0; i < 9; ++i) F[warp][i][lane] = i < 3 ? t[i] - tr : t[i];
+    }
+    __syncthreads();
+    if (!ok || warp > 1) return;
+    // planes (0,1) (0,2) (0,3) (1,2) (1,3) (2,3) are warps 0..5
+    const double sg = warp == 0 ? -1.0 : 1.0, hk = 0.5 * ck;
+    double gx[9], gy[9], gz[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        gx[i] = hk * fma(sg, F[2][i][lane], F[3][i][lane]);
+        gy[i] = hk * fma(sg, F[4][i][lane], -F[1][i][lane]);
+        gz[i] = hk * fma(sg, F[5][i][lane], F[0][i][lane]);
+    }
+    double s[36];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        s[i] = 0.5 + gz[i];
+        s[3 + i] = 0.5 - gz[i];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            // (a, b) element of G: diagonal real, upper triangle stored, lower its conjugate
+            auto el = [&](const double (&m)[9], double& re, double& im) {
+                const int lo = i < j ? i : j, hi = i < j ? j : i, q = 3 + 2 * (lo + hi - 1);
+                re = i == j ? m[i] : m[i == j ? 0 : q];
+                im = i == j ? 0.0 : i < j ? m[i == j ? 0 : q + 1] : -m[i == j ? 0 : q + 1];
+            };
+            double xr, xi, yr, yi, zr, zi;
+            el(gx, xr, xi);
+            el(gy, yr, yi);
+            el(gz, zr, zi);
+            if (i < j) {
+                s[tri(i, j)] = zr;
+                s[tri(i, j) + 1] = zi;
+                s[tri(3 + i, 3 + j)] = -zr;
+                s[tri(3 + i, 3 + j) + 1] = -zi;
+            }
+            s[tri(i, 3 + j)] = xr + yi;       // G_x - i G_y
+            s[tri(i, 3 + j) + 1] = xi - yr;
+        }
+    }
+    store_chiral(p == 0 ? fwd_e : fwd_o, g.Vh, h, warp, s);
+    double r[36];
+#pragma unroll
+    for (int i = 0; i < 36; ++i) r[i] = s[i];
+    if (!sweep_inverse(r)) {
+        double in[36], out[36];
+        for (int i = 0; i < 36; ++i) in[i] = s[i];
+        if (!invert_pivoted(in, out)) atomicExch(singular, 1);
+        else
+            for (int i = 0; i < 36; ++i) r[i] = out[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 36; ++i) r[i] *= 0.25;
+    store_chiral(p == 0 ? inv_e : inv_o, g.Vh, h, warp, r);
 }
 
 }  // namespace
@@ -203,7 +409,7 @@ __global__ void __launch_bounds__(128) k_clover_build(Geom g, const double* U, d
 // (Re)build the FP64 clover blocks of the handle's gauge field; lower-precision
 // copies are dropped and rebuilt on first use.
 int clover_build(wd_handle* h) {
-    const size_t bytes = (size_t)h->g.Vh * 144 * 16;
+    const size_t bytes = (size_t)h->g.Vh * 40 * 16;
     uint4* b[4];
     const char* names[4] = {"clov.fwd64.e", "clov.fwd64.o", "clov.inv64.e", "clov.inv64.o"};
     for (int i = 0; i < 4; ++i) {
@@ -213,42 +419,47 @@ int clover_build(wd_handle* h) {
     int* sing = (int*)workspace(h, "clov.singular", sizeof(int));
     if (!sing) return fail(h, WD_ERR_CUDA, "out of device memory");
     WD_CUDA(h, cudaMemset(sing, 0, sizeof(int)));
-    const long long V = 2LL * h->g.Vh;
-    const int grid = (int)std::min<long long>((V + 127) / 128, (long long)num_sms() * 16);
-    k_clover_build<<<grid, 128>>>(h->g, h->U64, h->csw * h->kappa, b[0], b[1], b[2], b[3], sing);
+    Field f{h->U64, {nullptr, nullptr}, 2LL * h->g.Vh, h->g.Vh};
+    if (h->fixed64) {   // SU(3) links: the products in fixed point, from the gathered FP64 links
+        const int rc = ensure_links(h, WD_FP64, 18, &f.l[0], &f.l[1]);
+        if (rc != WD_OK) return rc;
+    }
+    const dim3 grid((h->g.Vh + 31) / 32, 2);
+    const double ck = h->csw * h->kappa;
+    if (h->fixed64) k_clover_build<true><<<grid, 192>>>(h->g, f, ck, b[0], b[1], b[2], b[3], sing);
+    else k_clover_build<false><<<grid, 192>>>(h->g, f, ck, b[0], b[1], b[2], b[3], sing);
     WD_CUDA(h, cudaGetLastError());
     int hs = 0;
     WD_CUDA(h, cudaMemcpy(&hs, sing, sizeof(int), cudaMemcpyDeviceToHost));
     if (hs) return fail(h, WD_ERR_INVALID_ARG, "wd_set_clover: a clover block is singular");
     for (int k = 0; k < 2; ++k)
         for (int p = 0; p < 4; ++p) h->clov[k][p][0] = h->clov[k][p][1] = nullptr;
-    h->clov_inv64[0] = b[2];
-    h->clov_inv64[1] = b[3];
-    h->clov[1][WD_FP64][0] = b[0];
-    h->clov[1][WD_FP64][1] = b[1];
+    for (int p = 0; p < 2; ++p) {
+        h->clov64[1][p] = b[p];
+        h->clov64[0][p] = b[2 + p];
+    }
     h->gen += 1;
     return WD_OK;
 }
 
-// Clover blocks of kind 0 (C^{-1}) or 1 (C) in precision prec for both
-// parities; null pointers when the handle has no clover term.
+// Clover blocks of kind 0 (C^{-1}) or 1 (C) in precision prec (chiral packing)
+// for both parities; null pointers when the handle has no clover term.
 int ensure_clover(wd_handle* h, int prec, int kind, const uint4** even, const uint4** odd) {
     *even = *odd = nullptr;
     if (!h->have_clover) return WD_OK;
     for (int p = 0; p < 2; ++p) {
-        if (!h->clov[kind][prec][p]) {
-            // C^-1: chiral packing, 80 reals per site; C: full block, 288 reals per site
-            const size_t per_unit = 16 / (prec == WD_FP64 ? 8 : prec == WD_FP32 ? 4 : 2);
-            const size_t units = (kind == 0 ? 80 : 288) / per_unit;
+        if (prec == WD_FP64) {
+            h->clov[kind][prec][p] = h->clov64[kind][p];
+        } else if (!h->clov[kind][prec][p]) {
+            const size_t units = 80 / (prec == WD_FP32 ? 4 : 2 * 4);
             const std::string name = "clov.k" + std::to_string(kind) + ".p" + std::to_string(prec) + "." +
                                      std::to_string(p);
             uint4* dst = (uint4*)workspace(h, name, (size_t)h->g.Vh * units * 16);
             if (!dst) return fail(h, WD_ERR_CUDA, "out of device memory (clover blocks)");
-            const uint4* src = kind == 0 ? h->clov_inv64[p] : h->clov[1][WD_FP64][p];
+            const uint4* src = h->clov64[kind][p];
             cudaError_t e = by_prec(prec, [&](auto tag) {
                 typedef typename decltype(tag)::type T;
-                return kind == 0 ? Ops<T>::chiral_from64(h->g.Vh, src, dst, nullptr)
-                                 : Ops<T>::mat_from64(h->g.Vh, src, dst, nullptr);
+                return Ops<T>::chiral_from64(h->g.Vh, src, dst, nullptr);
             });
             WD_CUDA(h, e);
             WD_CUDA(h, cudaDeviceSynchronize());
@@ -274,7 +485,6 @@ extern "C" int wd_set_clover(wd_handle* h, double csw) {
         h->csw = 0.0;
         for (int k = 0; k < 2; ++k)
             for (int p = 0; p < 4; ++p) h->clov[k][p][0] = h->clov[k][p][1] = nullptr;
-        h->clov_inv64[0] = h->clov_inv64[1] = nullptr;
         h->gen += 1;
         return WD_OK;
     }

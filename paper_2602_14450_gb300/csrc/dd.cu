@@ -269,11 +269,8 @@ int wd_dd_set_partition(wd_handle* h, const int grid[4], const int coords[4]) {
     for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 2; ++b)
             for (int c = 0; c < 2; ++c)
-                if (h->links[a][b][c]) {
-                    cudaDeviceSynchronize();
-                    cudaFree(h->links[a][b][c]);
-                    h->links[a][b][c] = nullptr;
-                }
+                h->links[a][b][c] = nullptr;
+    WD_CUDA(h, cudaDeviceSynchronize());   // they are rewritten in place
     h->gen += 1;
     return WD_OK;
 }

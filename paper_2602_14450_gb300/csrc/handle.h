@@ -39,7 +39,8 @@ struct wd_handle {
     bool have_gauge = false;
     double unit_dev = -1.0, det_dev = -1.0;
     bool fixed64 = false;              // the FP64 18-real links are held as fixed-point digits (SU(3) links)
-    uint4* links[4][2][2] = {};        // [prec][recon 12 -> 0, 18 -> 1][output parity]
+    uint4* links[4][2][2] = {};        // [prec][recon 12 -> 0, 18 -> 1][output parity], null until built
+    uint4* link_buf[4][2][2] = {};     // their memory, kept when a new gauge field makes them stale
 
     std::map<std::string, Buffer> ws; // named device workspaces
     long long gen = 0;                 // bumped whenever a workspace moves
@@ -61,8 +62,8 @@ struct wd_handle {
 
     double csw = 0.0;                  // clover coefficient of wd_set_clover (0: plain Wilson)
     bool have_clover = false;
-    uint4* clov[2][4][2] = {};         // clover blocks [C^-1 (chiral packing), C (full)][prec][parity], on first use
-    uint4* clov_inv64[2] = {};         // full FP64 C^-1 per parity, the source of the chiral packings
+    uint4* clov64[2][2] = {};          // clover blocks [C^-1, C][parity] in FP64, chiral packing, of the gauge field
+    uint4* clov[2][4][2] = {};         // the blocks an operator of a precision uses, made from them on first use
 
     // hop kernel chosen by wd_tune per [prec][recon 12 -> 0, 18 -> 1][without / with fused reduction]; 0 = default
     int tune_variant[4][2][2] = {};

@@ -278,13 +278,6 @@ cudaError_t Ops<T>::hop(int recon, int epi, int red, const HopParams& P, cudaStr
 }
 
 template <typename T>
-cudaError_t Ops<T>::apply_mat(int n, int nrhs, long long vs, const uint4* mat, const uint4* in, uint4* out,
-                              cudaStream_t s) {
-    k_apply_mat<T><<<stream_blocks(n, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, mat, in, out);
-    return cudaGetLastError();
-}
-
-template <typename T>
 cudaError_t Ops<T>::apply_chiral(int n, int nrhs, long long vs, const uint4* mat, const uint4* in, uint4* out,
                                  cudaStream_t s) {
     k_apply_chiral<T><<<stream_blocks(n, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, mat, in, out);
@@ -293,13 +286,7 @@ cudaError_t Ops<T>::apply_chiral(int n, int nrhs, long long vs, const uint4* mat
 
 template <typename T>
 cudaError_t Ops<T>::chiral_from64(int n, const uint4* src64, uint4* dst, cudaStream_t s) {
-    k_chiral_from64<T><<<stream_blocks(n, 128), 128, 0, s>>>(n, src64, dst);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t Ops<T>::mat_from64(int n, const uint4* src64, uint4* dst, cudaStream_t s) {
-    k_mat_from64<T><<<stream_blocks(n, VEC_BLOCK), VEC_BLOCK, 0, s>>>(n, src64, dst);
+    k_chiral_from64<T><<<dim3(stream_blocks(n, VEC_BLOCK), 80 / Unit<T>::N), VEC_BLOCK, 0, s>>>(n, src64, dst);
     return cudaGetLastError();
 }
 
@@ -391,12 +378,17 @@ cudaError_t Ops<T>::unpack(const Geom& g, int parity, const uint4* in, double* l
 template <typename T>
 cudaError_t Ops<T>::build_links(int recon, const Geom& g, int parity, const double* U, uint4* out, bool fixed64,
                                 cudaStream_t s) {
+    const auto grid = [&](int links) { return dim3(stream_blocks(g.Vh, VEC_BLOCK), 8 / links); };
+    if constexpr (std::is_same<T, double>::value) {
+        if (recon == 18 && fixed64) {
+            k_build_links<T, 18, true><<<grid(LinkGroup<T, 18>::G), VEC_BLOCK, 0, s>>>(g, parity, U, out);
+            return cudaGetLastError();
+        }
+    }
     if (recon == 12)
-        k_build_links<T, 12, false><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
-    else if (recon == 18 && fixed64 && std::is_same<T, double>::value)
-        k_build_links<T, 18, true><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
+        k_build_links<T, 12, false><<<grid(LinkGroup<T, 12>::G), VEC_BLOCK, 0, s>>>(g, parity, U, out);
     else if (recon == 18)
-        k_build_links<T, 18, false><<<stream_blocks(g.Vh, VEC_BLOCK), VEC_BLOCK, 0, s>>>(g, parity, U, out);
+        k_build_links<T, 18, false><<<grid(LinkGroup<T, 18>::G), VEC_BLOCK, 0, s>>>(g, parity, U, out);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();

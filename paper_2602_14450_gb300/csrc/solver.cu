@@ -563,10 +563,10 @@ int solve_systems(int n, wd_handle* const* hs, const int* nrhs, const double* co
             WD_CUDA(h, Ops<double>::apply_chiral(nv, S.nrhs, S.vs64, S.mi64o, S.eta_o, S.xo, s));
             WD_CUDA(h, hop64(S, 1, S.x64, S.xo, EPI_Y, RED_NONE, kap, S.xo, 1.0, nullptr, 0.0, ST_NONE, GUARD_NONE, s,
                              S.mi64o));
-            WD_CUDA(h, Ops<double>::apply_mat(nv, S.nrhs, S.vs64, S.mf64e, S.x64, S.r64, s));
+            WD_CUDA(h, Ops<double>::apply_chiral(nv, S.nrhs, S.vs64, S.mf64e, S.x64, S.r64, s));
             WD_CUDA(h, hop64(S, 0, S.xo, S.r64, EPI_YZ, RED_NORM, kap, S.eta_e, 1.0, S.r64, -1.0, ST_ACC_SET,
                              GUARD_NONE, s));
-            WD_CUDA(h, Ops<double>::apply_mat(nv, S.nrhs, S.vs64, S.mf64o, S.xo, S.tmp64, s));
+            WD_CUDA(h, Ops<double>::apply_chiral(nv, S.nrhs, S.vs64, S.mf64o, S.xo, S.tmp64, s));
             WD_CUDA(h, hop64(S, 1, S.x64, S.tmp64, EPI_YZ, RED_NORM, kap, S.eta_o, 1.0, S.tmp64, -1.0, ST_ACC,
                              GUARD_NONE, s));
             nk += 3;
