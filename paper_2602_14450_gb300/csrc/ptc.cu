@@ -14,8 +14,9 @@
 // then W2[k][c][s][t][re,im], 9 * 12 * 16 complex each. The kernels read them
 // as given (the library stores BF16-rounded values for the solver).
 //
-// Training kernels compute, for L = sum |M v - y|^2/|y|^2 + mu |A M v - v|^2/|v|^2,
-// the weight gradients dL/dRe W + i dL/dIm W by the adjoint network.
+// Training: for L = sum |M v - y|^2/|y|^2 + mu |A M v - v|^2/|v|^2 the weight
+// gradients dL/dRe W + i dL/dIm W follow from the 8 x 8 (+ 1) correlations of
+// the transported loss gradient with the transported input (below).
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -97,110 +98,6 @@ __device__ __forceinline__ void spin_mul_add(const float2* w, const float (&phi)
     spin_mul_add_p(w, phi, acc);
 }
 
-// T_k f at site h of parity p, f read from the parity its support lives on.
-// Returns false when that source parity holds no data.
-template <typename TF, typename LT, int R>
-__device__ __forceinline__ bool transported(const Geom& g, int p, int h, const Coord& c, int k, const uint4* f_same,
-                                            const uint4* f_other, const uint4* links_p, float (&phi)[24]) {
-    if (k == 0) {
-        if (!f_same) return false;
-        load_spinor<TF>(f_same, g.Vh, h, phi);
-        return true;
-    }
-    if (!f_other) return false;
-    const int d = k - 1;
-    bool wrap;
-    const int hn = neighbour(g, h, c, d, &wrap);
-    float f[24], m[18];
-    load_spinor<TF>(f_other, g.Vh, hn, f);
-    if (wrap && g.bc[d >> 1] < 0) {
-#pragma unroll
-        for (int i = 0; i < 24; ++i) f[i] = -f[i];
-    }
-    load_link<LT, R>(links_p, g.Vh, h, d, m);
-    colour_mul(m, f, phi);
-    return true;
-}
-
-__device__ __forceinline__ const uint4* H_channel(const uint4* H, long long hvs, int c, int p) {
-    return H + (size_t)(2 * c + p) * hvs;
-}
-
-// Fan-out layer: one input channel (per-parity pointers, null = zero) to
-// channel blockIdx.y of H on parity blockIdx.z. H layout: [c][parity][units][Vh].
-template <typename TIN, typename TH, typename LT, int R>
-__global__ void __launch_bounds__(128) k_ptc_fanout(Geom g, const uint4* in_e, const uint4* in_o, uint4* H,
-                                                    long long hvs, const uint4* links_e, const uint4* links_o,
-                                                    const float* w, const SolverState* guard) {
-    if (guarded(guard, GUARD_INNER)) return;
-    __shared__ float2 ws[9 * 16];
-    const int c = blockIdx.y, p = blockIdx.z;
-    for (int i = threadIdx.x; i < 9 * 16; i += blockDim.x) {
-        const int k = i / 16, e = i % 16;
-        ws[i] = make_float2(w[2 * ((k * PTC_C + c) * 16 + e)], w[2 * ((k * PTC_C + c) * 16 + e) + 1]);
-    }
-    __syncthreads();
-    const uint4* same = p == 0 ? in_e : in_o;
-    const uint4* other = p == 0 ? in_o : in_e;
-    const uint4* links = p == 0 ? links_e : links_o;
-    uint4* out = H + (size_t)(2 * c + p) * hvs;
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += gridDim.x * blockDim.x) {
-        const Coord co = coord_of(g, p, h);
-        float acc[24];
-#pragma unroll
-        for (int i = 0; i < 24; ++i) acc[i] = 0.f;
-#pragma unroll 1
-        for (int k = 0; k < 9; ++k) {
-            float phi[24];
-            if (transported<TIN, LT, R>(g, p, h, co, k, same, other, links, phi)) spin_mul_add(&ws[16 * k], phi, acc);
-        }
-        store_spinor<TH>(out, g.Vh, h, acc);
-    }
-}
-
-// Fan-in layer: the 12 channels of H to one output channel on the even sites.
-template <typename TH, typename TOUT, typename LT, int R>
-__global__ void __launch_bounds__(128) k_ptc_fanin(Geom g, const uint4* H, long long hvs, uint4* out_e,
-                                                   const uint4* links_e, const float* w, const SolverState* guard) {
-    if (guarded(guard, GUARD_INNER)) return;
-    __shared__ float2 ws[9 * PTC_C * 16];
-    for (int i = threadIdx.x; i < 9 * PTC_C * 16; i += blockDim.x) ws[i] = make_float2(w[2 * i], w[2 * i + 1]);
-    __syncthreads();
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += gridDim.x * blockDim.x) {
-        const Coord co = coord_of(g, 0, h);
-        float acc[24];
-#pragma unroll
-        for (int i = 0; i < 24; ++i) acc[i] = 0.f;
-#pragma unroll 1
-        for (int k = 0; k < 9; ++k) {
-            float m[18];
-            int hn = h;
-            bool wrap = false;
-            if (k > 0) {
-                hn = neighbour(g, h, co, k - 1, &wrap);
-                load_link<LT, R>(links_e, g.Vh, h, k - 1, m);
-            }
-            const float ph = (wrap && g.bc[(k - 1) >> 1] < 0) ? -1.f : 1.f;
-#pragma unroll 1
-            for (int c = 0; c < PTC_C; ++c) {
-                const uint4* src = H + (size_t)(2 * c + (k == 0 ? 0 : 1)) * hvs;
-                float f[24], phi[24];
-                load_spinor<TH>(src, g.Vh, hn, f);
-                if (k == 0) {
-#pragma unroll
-                    for (int i = 0; i < 24; ++i) phi[i] = f[i];
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 24; ++i) f[i] *= ph;
-                    colour_mul(m, f, phi);
-                }
-                spin_mul_add(&ws[16 * (k * PTC_C + c)], phi, acc);
-            }
-        }
-        store_spinor<TOUT>(out_e, g.Vh, h, acc);
-    }
-}
-
 // ---------------------------------------------------------- collapsed M ---
 //
 // The network has no nonlinearity and its spin weights commute with the
@@ -210,8 +107,7 @@ __global__ void __launch_bounds__(128) k_ptc_fanin(Geom g, const uint4* H, long 
 // For an even-site input (odd sites zero) only phi_0 = V[0][0] psi on the
 // even sites and phi_{1+d} (d = 0..7) on the odd sites are nonzero, so M is
 // two stencil passes with eight odd-site intermediate fields instead of the
-// twelve hidden channels on both parities. The layered kernels above stay for
-// training, which needs the hidden activations.
+// twelve hidden channels on both parities.
 
 // V[k2][k1][s][t] from the BF16-rounded weights (double accumulation).
 __global__ void k_ptc_collapse(const float* w, float2* V) {
@@ -241,6 +137,8 @@ template <typename TIN, typename TPHI, typename LT, int R>
 __global__ void __launch_bounds__(128) k_ptc_s1(Geom g, const uint4* in_e, uint4* phi, long long pvs,
                                                 const uint4* links_o, const float2* V, const SolverState* guard) {
     if (guarded(guard, GUARD_INNER)) return;
+    in_e += blockIdx.y * (long long)Spinor<TIN>::UNITS * g.Vh;      // sample blockIdx.y, vectors back to back
+    phi += blockIdx.y * 8 * pvs;
     __shared__ float ts[S1_SITES * S1_STRIDE];
     __shared__ float2 vs[8 * S1_VROW];
     for (int i = threadIdx.x; i < 64 * 16; i += blockDim.x) {
@@ -375,6 +273,9 @@ __global__ void __launch_bounds__(128) k_ptc_s2(Geom g, const uint4* in_e, const
                                                 uint4* out_e, const uint4* links_e, const float2* V,
                                                 const SolverState* guard) {
     if (guarded(guard, GUARD_INNER)) return;
+    in_e += blockIdx.y * (long long)Spinor<TIN>::UNITS * g.Vh;      // sample blockIdx.y, as in k_ptc_s1
+    phi += blockIdx.y * 8 * pvs;
+    out_e += blockIdx.y * (long long)Spinor<TOUT>::UNITS * g.Vh;
     __shared__ float2 v00[16];
     if (threadIdx.x < 16) v00[threadIdx.x] = V[threadIdx.x];
     __syncthreads();
@@ -418,127 +319,257 @@ __global__ void __launch_bounds__(128) k_ptc_s2(Geom g, const uint4* in_e, const
 
 namespace wd {
 
-// Weight gradient: dW[k][c] += sum_x sum_colour G_c(x) (x) conj(T_k F_c(x)), summed into
-// grad (float, [k][c][s][t][re,im]). Mode 0 (layer 2): G = one even channel,
-// F = the channels of H. Mode 1 (layer 1): G = the channels of H-shaped g_H,
-// F = one even channel. One block row per (k, c) = (blockIdx.y, blockIdx.z).
-template <typename LT, int R>
-__global__ void __launch_bounds__(128) k_ptc_wgrad(Geom g, int mode, const uint4* G, const uint4* F, long long hvs,
-                                                   const uint4* links_e, const uint4* links_o, float* part) {
-    const int k = blockIdx.y, c = blockIdx.z;
+// --------------------------------------------------------------- training ---
+//
+// With g = 2 dL/dconj(M v) on the even sites, the gradients of both layers are
+// small products of the weights with one set of 4 x 4 spin matrices,
+//   C[k][k'] = sum over sites and colours of (T_kbar g) (x) conj(T_k' v),  kbar the opposite hop of k,
+//   dW2[k][c] = sum_k' C[k][k'] W1[k'][c]^+,   dW1[k'][c] = sum_k W2[k][c]^+ C[k][k'],
+// because the hidden channels are H_c = sum_k' W1[k'][c] T_k' v and a transport
+// moves from one side of the colour contraction to the other as its adjoint.
+// The transports of v and g live on the odd sites (k, k' = 1..8), k = k' = 0 on
+// the even ones; all other C vanish. So no hidden channel is formed: M v comes
+// from the collapsed network and C is one contraction over 3 V/2 (site, colour)
+// rows with 32 x 32 complex results.
+
+constexpr int CORR_SITES = 32;                       // odd sites per tile
+constexpr int CORR_ROW = 34;                         // complex numbers per tile row (32, padded: conflict-free writes)
+constexpr int CORR_SMEM = 2 * 3 * CORR_SITES * CORR_ROW * (int)sizeof(float2);
+constexpr int CORR_FLOATS = 2 * 32 * 32;             // C[1 + d][1 + d'][s][t] as rows (d, s), columns (d', t)
+
+// C over the odd sites of nb samples, each block's sum to its own slot of
+// `part`. Per tile of 32 sites warp mu computes directions 2 mu and 2 mu + 1 of
+// both fields (the link and the neighbour index once for both) into shared
+// memory as rows (site, colour) x 32 complex; then 64 threads per half of the
+// rows hold 4 x 4 complex results each in registers. Bound by the FP32 pipe:
+// 14.6k multiply-adds per site and sample.
+__global__ void __launch_bounds__(128, 4) k_ptc_corr(Geom g, int nb, const uint4* v, const uint4* gr, long long vs,
+                                                     const uint4* links_o, float* part) {
+    extern __shared__ __align__(16) unsigned char corr_smem[];
+    float2* A = reinterpret_cast<float2*>(corr_smem);               // T_kbar g: column 4 d + s
+    float2* B = A + 3 * CORR_SITES * CORR_ROW;                      // T_k' v: column 4 d' + t
+    const int tid = threadIdx.x, mu = tid >> 5, lane = tid & 31;
+    const int half = tid >> 6, r = (tid & 63) >> 3, c = tid & 7;
+    float re[4][4], im[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) re[i][j] = im[i][j] = 0.f;
+    const int tiles = (g.Vh + CORR_SITES - 1) / CORR_SITES;
+    for (int t = blockIdx.x; t < nb * tiles; t += gridDim.x) {
+        const int sample = t / tiles, h = (t - sample * tiles) * CORR_SITES + lane;
+        const uint4 *vi = v + sample * vs, *gi = gr + sample * vs;
+        const bool ok = h < g.Vh;
+        const Coord co = ok ? coord_of(g, 1, h) : Coord{};
+#pragma unroll 1
+        for (int j = 0; j < 2; ++j) {
+            const int d = 2 * mu + j;
+            float fv[24], fg[24];
+            if (ok) {
+                bool wrap;
+                const int hn = neighbour(g, h, co, d, &wrap);
+                float f[24], m[18];
+                load_link<float, 18>(links_o, g.Vh, h, d, m);
+                if (wrap && g.bc[mu] < 0) {
+#pragma unroll
+                    for (int i = 0; i < 18; ++i) m[i] = -m[i];
+                }
+                load_spinor<float>(vi, g.Vh, hn, f);
+                colour_mul(m, f, fv);
+                load_spinor<float>(gi, g.Vh, hn, f);
+                colour_mul(m, f, fg);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 24; ++i) fv[i] = fg[i] = 0.f;
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                float4* pb = reinterpret_cast<float4*>(B + (3 * lane + a) * CORR_ROW + 4 * d);
+                float4* pa = reinterpret_cast<float4*>(A + (3 * lane + a) * CORR_ROW + 4 * (d ^ 1));
+#pragma unroll
+                for (int s = 0; s < 4; s += 2) {
+                    const int e = 2 * (3 * s + a), e2 = e + 6;
+                    pb[s / 2] = make_float4(fv[e], fv[e + 1], fv[e2], fv[e2 + 1]);
+                    pa[s / 2] = make_float4(fg[e], fg[e + 1], fg[e2], fg[e2 + 1]);
+                }
+            }
+        }
+        __syncthreads();
+        const float4* pa = reinterpret_cast<const float4*>(A + half * 48 * CORR_ROW + 4 * r);
+        const float4* pb = reinterpret_cast<const float4*>(B + half * 48 * CORR_ROW + 4 * c);
+#pragma unroll 2
+        for (int k = 0; k < 48; ++k, pa += CORR_ROW / 2, pb += CORR_ROW / 2) {
+            const float4 a0 = pa[0], a1 = pa[1], b0 = pb[0], b1 = pb[1];
+            const float ar[4] = {a0.x, a0.z, a1.x, a1.z}, ai[4] = {a0.y, a0.w, a1.y, a1.w};
+            const float br[4] = {b0.x, b0.z, b1.x, b1.z}, bi[4] = {b0.y, b0.w, b1.y, b1.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {   // a conj(b)
+                    re[i][j] = __fmaf_rn(ai[i], bi[j], __fmaf_rn(ar[i], br[j], re[i][j]));
+                    im[i][j] = __fmaf_rn(-ar[i], bi[j], __fmaf_rn(ai[i], br[j], im[i][j]));
+                }
+        }
+        __syncthreads();
+    }
+    float4* sum = reinterpret_cast<float4*>(corr_smem) + 8 * (tid & 63);   // the second half's share
+    if (half == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            sum[2 * i] = make_float4(re[i][0], im[i][0], re[i][1], im[i][1]);
+            sum[2 * i + 1] = make_float4(re[i][2], im[i][2], re[i][3], im[i][3]);
+        }
+    }
+    __syncthreads();
+    if (half == 0) {
+        float4* out = reinterpret_cast<float4*>(part + (size_t)blockIdx.x * CORR_FLOATS);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float4 w = sum[2 * i + q];
+                out[(4 * r + i) * 16 + 2 * c + q] =
+                    make_float4(re[i][2 * q] + w.x, im[i][2 * q] + w.y, re[i][2 * q + 1] + w.z, im[i][2 * q + 1] + w.w);
+            }
+    }
+}
+
+// sum[i] (+)= sum over blocks of part[block][i] for `n` floats a block, in a fixed order, as FP32 pairs.
+__global__ void __launch_bounds__(256) k_ptc_corr_sum(int blocks, int n, const float* part, int add, float* sum) {
+    __shared__ float2 sh[8][32];
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31), q = threadIdx.x >> 5;
+    F2 t = {0.f, 0.f};
+#pragma unroll 4
+    for (int b = q; b < blocks; b += 8) t = f2_add(t, F2{part[(size_t)b * n + i], 0.f});
+    sh[q][threadIdx.x & 31] = make_float2(t.hi, t.lo);
+    __syncthreads();
+    if (q == 0) {
+        if (add) t = f2_add(t, F2{sum[i], 0.f});
+        for (int w = 1; w < 8; ++w) t = f2_add(t, F2{sh[w][threadIdx.x].x, sh[w][threadIdx.x].y});
+        sum[i] = t.hi;
+    }
+}
+
+// Gradients of both layers from C (rows (d, s), columns (d', t)) and C[0][0] (4 x 4): one complex element a thread.
+__global__ void k_ptc_wgrad(const float2* C, const float2* C00, const float2* w, float2* grad) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 2 * PTC_LAYER) return;
+    const int layer = i / PTC_LAYER, e = i % PTC_LAYER;
+    const int k = e / (PTC_C * 16), c = (e / 16) % PTC_C, s = (e / 4) % 4, t = e % 4;
+    const float2* w1 = w + c * 16;                   // W1[k'][c] at + k' PTC_C 16
+    const float2* w2 = w + PTC_LAYER + c * 16;
+    float re = 0.f, im = 0.f;
+    const int n = k == 0 ? 1 : 8;
+    for (int q = 0; q < n; ++q) {
+        const int kq = k == 0 ? 0 : 1 + q;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float2 a, b;                             // += a conj(b)
+            if (layer == 1) {                        // dW2[k][s][t] = sum C[k][k'][s][u] conj(W1[k'][t][u])
+                a = k == 0 ? C00[4 * s + u] : C[(4 * (k - 1) + s) * 32 + 4 * q + u];
+                b = w1[kq * PTC_C * 16 + 4 * t + u];
+            } else {                                 // dW1[k'][s][t] = sum conj(W2[k][u][s]) C[k][k'][u][t]
+                a = k == 0 ? C00[4 * u + t] : C[(4 * q + u) * 32 + 4 * (k - 1) + t];
+                b = w2[kq * PTC_C * 16 + 4 * u + s];
+            }
+            re = __fmaf_rn(a.x, b.x, __fmaf_rn(a.y, b.y, re));
+            im = __fmaf_rn(a.y, b.x, __fmaf_rn(-a.x, b.y, im));
+        }
+    }
+    grad[i] = make_float2(re, im);
+}
+
+// x^2 added to the FP32 pair s: the square's rounding error is kept.
+__device__ __forceinline__ void add_square(F2& s, float x) {
+    const float p = __fmul_rn(x, x);
+    s = f2_add(s, F2{p, __fmaf_rn(x, x, -p)});
+}
+
+// For sample blockIdx.y: t = gamma5 e2 with e2 = a - v (a = A m), and this
+// block's share of |v|^2, |y|^2, |m - y|^2, |e2|^2 (FP32 pairs, about 48 bits).
+__global__ void __launch_bounds__(256) k_ptc_resid(int Vh, long long vs, const float4* v, const float4* y,
+                                                   const float4* m, const float4* a, float4* t, double* part) {
+    const long long o = blockIdx.y * vs;
+    F2 s[4] = {};
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < vs; i += (long long)gridDim.x * blockDim.x) {
+        const float4 vv = v[o + i], yv = y[o + i], mv = m[o + i], av = a[o + i];
+        const float4 e1 = make_float4(mv.x - yv.x, mv.y - yv.y, mv.z - yv.z, mv.w - yv.w);
+        const float4 e2 = make_float4(av.x - vv.x, av.y - vv.y, av.z - vv.z, av.w - vv.w);
+        // (g5 f)_s = -f_{s xor 2}: spins 0, 1 are units 0..2 of a site, spins 2, 3 units 3..5
+        t[o + (i < vs / 2 ? i + vs / 2 : i - vs / 2)] = make_float4(-e2.x, -e2.y, -e2.z, -e2.w);
+        const float4 q[4] = {vv, yv, e1, e2};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            add_square(s[k], q[k].x);
+            add_square(s[k], q[k].y);
+            add_square(s[k], q[k].z);
+            add_square(s[k], q[k].w);
+        }
+    }
+    block_sum<4>(s);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 4; ++k)
+            part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + k] = (double)s[k].hi + (double)s[k].lo;
+}
+
+// dots[sample][4] = the sums of k_ptc_resid over its nb blocks, in a fixed order (one warp per sample).
+__global__ void k_ptc_dots(int nb, const double* part, double* dots) {
+    const double* p = part + (size_t)blockIdx.x * nb * 4;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nb; b += 32)
+        for (int k = 0; k < 4; ++k) s[k] += p[4 * b + k];
+    block_sum<4>(s);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 4; ++k) dots[4 * blockIdx.x + k] = s[k];
+}
+
+// g = 2 (m - y) / |y|^2 + 2 mu gamma5 b / |v|^2 (b = A gamma5 e2) for sample blockIdx.y, and this block's share of
+// C[0][0] = sum g (x) conj(v) over the even sites, 32 floats per block.
+__global__ void __launch_bounds__(128) k_ptc_lossgrad(int Vh, long long vs, const uint4* v, const uint4* y,
+                                                      const uint4* m, const uint4* b, const double* dots, double mu,
+                                                      uint4* gr, float* part) {
+    const long long o = blockIdx.y * vs;
+    const float cy = (float)(2.0 / dots[4 * blockIdx.y + 1]), cv = (float)(2.0 * mu / dots[4 * blockIdx.y]);
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-    for (int p = 0; p < 2; ++p) {
-        if (mode == 0 && p == 1) break;      // layer-2 output lives on even sites only
-        const uint4* links = p == 0 ? links_e : links_o;
-        const uint4* gsrc = mode == 0 ? G : G + (size_t)(2 * c + p) * hvs;
-        const uint4 *f_same, *f_other;
-        if (mode == 0) {
-            f_same = H_channel(F, hvs, c, p);
-            f_other = H_channel(F, hvs, c, 1 - p);
-        } else {
-            f_same = p == 0 ? F : nullptr;
-            f_other = p == 0 ? nullptr : F;
-        }
-        for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += gridDim.x * blockDim.x) {
-            const Coord co = coord_of(g, p, h);
-            float phi[24];
-            if (!transported<float, LT, R>(g, p, h, co, k, f_same, f_other, links, phi)) continue;
-            float gv[24];
-            load_spinor<float>(gsrc, g.Vh, h, gv);
+    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < Vh; h += gridDim.x * blockDim.x) {
+        float f[24], e[24], gv[24];
+        load_spinor<float>(m + o, Vh, h, e);
+        load_spinor<float>(y + o, Vh, h, f);
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
+        for (int i = 0; i < 24; ++i) gv[i] = cy * (e[i] - f[i]);
+        load_spinor<float>(b + o, Vh, h, f);
 #pragma unroll
-                for (int t = 0; t < 4; ++t)
+        for (int i = 0; i < 24; ++i) gv[i] = __fmaf_rn(-cv, f[(i + 12) % 24], gv[i]);
+        store_spinor<float>(gr + o, Vh, h, gv);
+        load_spinor<float>(v + o, Vh, h, f);
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {   // g_{s,a} conj(phi_{t,a})
-                        const float gr = gv[2 * (3 * s + a)], gi = gv[2 * (3 * s + a) + 1];
-                        const float fr = phi[2 * (3 * t + a)], fi = phi[2 * (3 * t + a) + 1];
-                        acc[2 * (4 * s + t)] += gr * fr + gi * fi;
-                        acc[2 * (4 * s + t) + 1] += gi * fr - gr * fi;
-                    }
-        }
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {   // g_{s,a} conj(v_{t,a})
+                    const float xr = gv[2 * (3 * s + a)], xi = gv[2 * (3 * s + a) + 1];
+                    const float yr = f[2 * (3 * t + a)], yi = f[2 * (3 * t + a) + 1];
+                    acc[2 * (4 * s + t)] = __fmaf_rn(xi, yi, __fmaf_rn(xr, yr, acc[2 * (4 * s + t)]));
+                    acc[2 * (4 * s + t) + 1] = __fmaf_rn(-xr, yi, __fmaf_rn(xi, yr, acc[2 * (4 * s + t) + 1]));
+                }
     }
-    // block sum of the 32 accumulators into this block's partial-sum slots (summed in block order later)
     __shared__ float sh[32][4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
-        float v = acc[i];
+        float x = acc[i];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) sh[i][warp] = v;
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
+        if (lane == 0) sh[i][warp] = x;
     }
     __syncthreads();
     if (threadIdx.x < 32) {
-        float v = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[threadIdx.x][w];
-        part[((size_t)(k * PTC_C + c) * gridDim.x + blockIdx.x) * 32 + threadIdx.x] = v;
-    }
-}
-
-// grad[(k, c)][32] += sum over the nb blocks of k_ptc_wgrad's partial sums, in block order (deterministic).
-__global__ void k_ptc_wgrad_sum(int nb, const float* part, float* grad) {
-    const int kc = blockIdx.x;   // k * PTC_C + c
-    float v = 0.f;
-    for (int b = 0; b < nb; ++b) v += part[((size_t)kc * nb + b) * 32 + threadIdx.x];
-    grad[2 * (kc * 16) + threadIdx.x] += v;
-}
-
-}  // namespace wd
-
-namespace wd {
-
-// ------------------------------------------------------------ small kernels ---
-
-// z = a x + b y over n floats (y may be null)
-__global__ void k_f32_lincomb(long long n, float a, const float* x, float b, const float* y, float* z) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        z[i] = a * x[i] + (y ? b * y[i] : 0.f);
-}
-
-// part[block] = this block's share of sum x_i y_i (double accumulation)
-__global__ void k_f32_dot(long long n, const float* x, const float* y, double* part) {
-    double s = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        s += (double)x[i] * (double)y[i];
-    double v[1] = {s};
-    block_sum<1>(v);
-    if (threadIdx.x == 0) part[blockIdx.x] = v[0];
-}
-
-// *out = sum of nb partial sums in block order (deterministic)
-__global__ void k_sum_partials(int nb, const double* part, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nb; ++b) s += part[b];
-        *out = s;
-    }
-}
-
-// gamma5 of the Dirac representation: (g5 f)_s = -f_{s xor 2}
-__global__ void k_gamma5_f32(int Vh, const uint4* in, uint4* out) {
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < Vh; h += gridDim.x * blockDim.x) {
-        float f[24], o[24];
-        load_spinor_cg<float>(in, Vh, h, f);
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-#pragma unroll
-            for (int j = 0; j < 6; ++j) o[6 * s + j] = -f[6 * (s ^ 2) + j];
-        store_spinor<float>(out, Vh, h, o);
-    }
-}
-
-// Fan-out weights of the adjoint of layer 2: Wa[k'][c] = W2[k][c]^+, k' the opposite hop of k.
-__global__ void k_ptc_adjoint_weights(const float* w2, float* wa) {
-    for (int i = threadIdx.x; i < PTC_LAYER; i += blockDim.x) {
-        const int k = i / (PTC_C * 16), c = (i / 16) % PTC_C, s = (i / 4) % 4, t = i % 4;
-        const int ka = k == 0 ? 0 : 1 + ((k - 1) ^ 1);
-        const int src = (k * PTC_C + c) * 16 + 4 * t + s;   // transpose
-        const int dst = (ka * PTC_C + c) * 16 + 4 * s + t;
-        wa[2 * dst] = w2[2 * src];
-        wa[2 * dst + 1] = -w2[2 * src + 1];                 // conjugate
+        float x = 0.f;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) x += sh[threadIdx.x][w];
+        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 32 + threadIdx.x] = x;
     }
 }
 
@@ -568,7 +599,7 @@ static int grid_for(int n, int block) {
 }
 
 struct PtcBufs {
-    float *w, *weff, *m, *v, *grad, *wadj;
+    float *w, *weff, *m, *v, *grad;
     float2* V;      // collapsed spin weights V[k2][k1][s][t] of weff
 };
 
@@ -579,24 +610,16 @@ static int ptc_bufs(wd_handle* h, PtcBufs* b) {
     b->m = (float*)workspace(h, "ptc.m", nb);
     b->v = (float*)workspace(h, "ptc.v", nb);
     b->grad = (float*)workspace(h, "ptc.grad", nb);
-    b->wadj = (float*)workspace(h, "ptc.wadj", nb / 2);
     b->V = (float2*)workspace(h, "ptc.V", sizeof(float2) * 81 * 16);
-    if (!b->w || !b->weff || !b->m || !b->v || !b->grad || !b->wadj || !b->V)
+    if (!b->w || !b->weff || !b->m || !b->v || !b->grad || !b->V)
         return fail(h, WD_ERR_CUDA, "out of device memory");
     return WD_OK;
 }
 
-// Hidden buffer of 12 channels x 2 parities in storage type of `prec`.
-static uint4* ptc_hidden(wd_handle* h, int prec, const char* name) {
-    return (uint4*)workspace(h, name, vec_bytes(h, prec) * 2 * PTC_C);
-}
-
-// M in = out: FP32 path (FP32 hidden, FP32 18-real links) or FP16 path
-// (BF16 hidden, FP16 12-real links), weights from `w` (device, flat layout).
 int* ptc_err(wd_handle* h);
 
-// Whether M (its first pass, and in training the fan-out layers) mixes channels
-// on the tensor cores (environment WD_PTC_TC=0 selects the FP32-core kernels).
+// Whether the first pass of the FP16 path of M mixes channels on the tensor
+// cores (environment WD_PTC_TC=0 selects the FP32-core kernel).
 static bool ptc_tensor_cores() {
     static int v = -1;
     if (v < 0) {
@@ -604,52 +627,6 @@ static bool ptc_tensor_cores() {
         v = (e && e[0] == '0') ? 0 : 1;
     }
     return v == 1;
-}
-
-// Training fan-out (FP32 input on the even sites, FP32 18-real links) into the
-// 12 hidden channels of H on both parities: the even sites (hop 0 only) on the
-// FP32 cores, the odd sites (the eight transports) on the tensor cores.
-static cudaError_t ptc_fanout_f32(wd_handle* h, const uint4* in_e, uint4* H, long long hvs, const uint4* le,
-                                  const uint4* lo, const float* w, cudaStream_t s, int* err) {
-    const Geom& g = h->g;
-    const int gx = grid_for(g.Vh, 128);
-    if (!ptc_tensor_cores()) {
-        k_ptc_fanout<float, float, float, 18><<<dim3(gx, PTC_C, 2), 128, 0, s>>>(g, in_e, nullptr, H, hvs, le, lo, w,
-                                                                               nullptr);
-        return cudaGetLastError();
-    }
-    k_ptc_fanout<float, float, float, 18><<<dim3(gx, PTC_C, 1), 128, 0, s>>>(g, in_e, nullptr, H, hvs, le, lo, w,
-                                                                           nullptr);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_ptc_fanout_odd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             tcf::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    const long long tiles = ((long long)g.Vh + tc::TILE_M - 1) / tc::TILE_M;
-    const long long tcap = (long long)num_sms() * 3;
-    const int gt = (int)(tiles < tcap ? tiles : tcap);
-    k_ptc_fanout_odd_tc<<<gt, 128, tcf::SMEM_BYTES, s>>>(g, in_e, H, hvs, lo, w, err, h->wait_rounds);
-    return cudaGetLastError();
-}
-
-cudaError_t ptc_apply_raw(wd_handle* h, int prec, const uint4* in_e, uint4* out_e, uint4* H, const float* w,
-                          const uint4* le, const uint4* lo, cudaStream_t s, const SolverState* guard) {
-    const Geom& g = h->g;
-    const int blk = 128, gx = grid_for(g.Vh, blk);
-    if (prec == WD_FP32) {
-        const long long hvs = (long long)spinor_units(WD_FP32) * g.Vh;
-        cudaError_t e = ptc_fanout_f32(h, in_e, H, hvs, le, lo, w, s, ptc_err(h));
-        if (e != cudaSuccess) return e;
-        k_ptc_fanin<float, float, float, 18><<<gx, blk, 0, s>>>(g, H, hvs, out_e, le, w + 2 * PTC_LAYER, guard);
-    } else {
-        const long long hvs = (long long)spinor_units(WD_BF16) * g.Vh;
-        k_ptc_fanout<__half, __nv_bfloat16, __half, 12><<<dim3(gx, PTC_C, 2), blk, 0, s>>>(g, in_e, nullptr, H, hvs,
-                                                                                         le, lo, w, guard);
-        k_ptc_fanin<__nv_bfloat16, __half, __half, 12><<<gx, blk, 0, s>>>(g, H, hvs, out_e, le, w + 2 * PTC_LAYER, guard);
-    }
-    return cudaGetLastError();
 }
 
 // Device flag raised by a kernel whose bounded wait gave up.
@@ -663,6 +640,20 @@ static uint4* ptc_phi(wd_handle* h, int prec) {
 }
 
 
+// M on n FP32 vectors back to back (PHI: 8 vectors each).
+static cudaError_t ptc_apply_f32(wd_handle* h, int n, const uint4* in_e, uint4* out_e, uint4* PHI, const float2* V,
+                                 const uint4* le, const uint4* lo, cudaStream_t s,
+                                 const SolverState* guard = nullptr) {
+    const Geom& g = h->g;
+    const long long groups = ((long long)g.Vh + S1_SITES - 1) / S1_SITES, cap = (long long)num_sms() * 6;
+    const long long pvs = (long long)spinor_units(WD_FP32) * g.Vh;
+    k_ptc_s1<float, float, float, 18><<<dim3((int)std::min(groups, cap), n), 128, 0, s>>>(g, in_e, PHI, pvs, lo, V,
+                                                                                          guard);
+    k_ptc_s2<float, float, float, float, 18, false><<<dim3(grid_for(g.Vh, 128), n), 128, 0, s>>>(
+        g, in_e, PHI, pvs, out_e, le, V, guard);
+    return cudaGetLastError();
+}
+
 cudaError_t ptc_apply_m(wd_handle* h, int prec, const uint4* in_e, uint4* out_e, uint4* PHI, const float2* V,
                         const uint4* le, const uint4* lo, cudaStream_t s, const SolverState* guard, int* err) {
     const Geom& g = h->g;
@@ -671,9 +662,7 @@ cudaError_t ptc_apply_m(wd_handle* h, int prec, const uint4* in_e, uint4* out_e,
     const int g1 = (int)(groups < cap ? groups : cap);
     const int g2 = grid_for(g.Vh, 128);
     if (prec == WD_FP32) {
-        const long long pvs = (long long)spinor_units(WD_FP32) * g.Vh;
-        k_ptc_s1<float, float, float, 18><<<g1, 128, 0, s>>>(g, in_e, PHI, pvs, lo, V, guard);
-        k_ptc_s2<float, float, float, float, 18, false><<<g2, 128, 0, s>>>(g, in_e, PHI, pvs, out_e, le, V, guard);
+        return ptc_apply_f32(h, 1, in_e, out_e, PHI, V, le, lo, s, guard);
     } else if (ptc_tensor_cores()) {
         const long long pvs = (long long)spinor_units(WD_BF16) * g.Vh;
         static bool attr = false;
@@ -698,12 +687,13 @@ cudaError_t ptc_apply_m(wd_handle* h, int prec, const uint4* in_e, uint4* out_e,
     return cudaGetLastError();
 }
 
-// FP32 even-odd operator A (or A^+ = g5 A g5) on FP32 18-real links.
-static cudaError_t apply_A_f32(wd_handle* h, const uint4* in, uint4* out, uint4* tmp, const uint4* le, const uint4* lo,
-                               cudaStream_t s) {
+// FP32 even-odd operator A (or A^+ = g5 A g5) on FP32 18-real links, n vectors back to back.
+static cudaError_t apply_A_f32(wd_handle* h, int n, const uint4* in, uint4* out, uint4* tmp, const uint4* le,
+                               const uint4* lo, cudaStream_t s) {
     HopParams P{};
     P.g = h->g;
-    P.nrhs = 1;
+    P.nrhs = n;
+    P.vs = (long long)spinor_units(WD_FP32) * h->g.Vh;
     P.parity = 1;
     P.links = lo;
     P.in = in;
@@ -721,6 +711,9 @@ static cudaError_t apply_A_f32(wd_handle* h, const uint4* in, uint4* out, uint4*
     return Ops<float>::hop(18, EPI_Y, RED_NONE, P, s);
 }
 
+// Bytes of workspace of a chunk of samples (13 vectors each); a larger batch goes through chunk by chunk.
+constexpr size_t PTC_CHUNK_BYTES = (size_t)2 << 30;
+
 int ptc_grad(wd_handle* h, int n, const float* v, const float* y, double mu, double* loss, cudaStream_t s) {
     PtcBufs B;
     int rc = ptc_bufs(h, &B);
@@ -729,76 +722,53 @@ int ptc_grad(wd_handle* h, int n, const float* v, const float* y, double mu, dou
     if ((rc = ensure_links(h, WD_FP32, 18, &le, &lo)) != WD_OK) return rc;
     const Geom& g = h->g;
     const size_t vb = vec_bytes(h, WD_FP32);
-    const long long nf = (long long)g.Vh * 24;
-    const long long hvs = (long long)spinor_units(WD_FP32) * g.Vh;
-    uint4* H = ptc_hidden(h, WD_FP32, "ptc.h32");
-    uint4* GH = ptc_hidden(h, WD_FP32, "ptc.gh32");
-    float* m = (float*)workspace(h, "ptc.vm", vb);
-    float* e1 = (float*)workspace(h, "ptc.ve1", vb);
-    float* am = (float*)workspace(h, "ptc.vam", vb);
-    float* t1 = (float*)workspace(h, "ptc.vt1", vb);
-    float* t2 = (float*)workspace(h, "ptc.vt2", vb);
-    float* gv = (float*)workspace(h, "ptc.vg", vb);
-    double* dots = (double*)workspace(h, "ptc.dots", sizeof(double) * (4 * n + 4));
-    const int blk = 256, gv1 = grid_for((int)std::min<long long>(nf, 1LL << 30), blk);
-    const dim3 wgrid(std::max(1, num_sms() / 8), 9, PTC_C);
-    // per-block partial sums of the dot products and of the weight gradients, summed in block order
-    double* dpart = (double*)workspace(h, "ptc.dpart", sizeof(double) * gv1);
-    float* wpart = (float*)workspace(h, "ptc.wpart", sizeof(float) * 32 * wgrid.x * 9 * PTC_C);
-    if (!H || !GH || !m || !e1 || !am || !t1 || !t2 || !gv || !dots || !dpart || !wpart)
+    const long long vs = (long long)spinor_units(WD_FP32) * g.Vh;   // 16-byte units of a vector
+    const int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)n, PTC_CHUNK_BYTES / (13 * vb)));
+    uint4* m = (uint4*)workspace(h, "ptc.vm", vb * chunk);
+    uint4* am = (uint4*)workspace(h, "ptc.vam", vb * chunk);
+    uint4* t1 = (uint4*)workspace(h, "ptc.vt1", vb * chunk);
+    uint4* t2 = (uint4*)workspace(h, "ptc.vt2", vb * chunk);
+    uint4* gv = (uint4*)workspace(h, "ptc.vg", vb * chunk);
+    uint4* phi = (uint4*)workspace(h, "ptc.phi32", vb * 8 * chunk);
+    const int rb = (int)std::max<long long>(1, std::min<long long>((vs + 255) / 256, 128));      // blocks per sample
+    const int gb = std::max(1, std::min((g.Vh + 127) / 128, std::max(1, 4 * num_sms() / chunk)));
+    const int cb = (int)std::min<long long>((long long)chunk * ((g.Vh + CORR_SITES - 1) / CORR_SITES), 4 * num_sms());
+    double* dots = (double*)workspace(h, "ptc.dots", sizeof(double) * 4 * (size_t)n);
+    double* dpart = (double*)workspace(h, "ptc.dpart", sizeof(double) * 4 * (size_t)rb * chunk);
+    float* cpart = (float*)workspace(h, "ptc.cpart", sizeof(float) * (size_t)CORR_FLOATS * cb);
+    float* c0part = (float*)workspace(h, "ptc.c0part", sizeof(float) * 32 * (size_t)gb * chunk);
+    float* C = (float*)workspace(h, "ptc.C", sizeof(float) * (CORR_FLOATS + 32));
+    if (!m || !am || !t1 || !t2 || !gv || !phi || !dots || !dpart || !cpart || !c0part || !C)
         return fail(h, WD_ERR_CUDA, "out of device memory");
-    auto dot = [&](const float* a, const float* b, double* out) {
-        k_f32_dot<<<gv1, blk, 0, s>>>(nf, a, b, dpart);
-        k_sum_partials<<<1, 32, 0, s>>>(gv1, dpart, out);
-    };
-    int* err = ptc_err(h);
-    if (!err) return fail(h, WD_ERR_CUDA, "out of device memory");
-    WD_CUDA(h, cudaMemsetAsync(err, 0, sizeof(int), s));
-    WD_CUDA(h, cudaMemsetAsync(dots, 0, sizeof(double) * (4 * n + 4), s));
-    WD_CUDA(h, cudaMemsetAsync(B.grad, 0, sizeof(float) * PTC_FLOATS, s));
-    // input norms first: the gradient coefficients need them
-    for (int i = 0; i < n; ++i) {
-        const float* vi = v + i * nf;
-        const float* yi = y + i * nf;
-        dot(vi, vi, dots + 4 * i);
-        dot(yi, yi, dots + 4 * i + 1);
+    static bool attr = false;
+    if (!attr) {
+        WD_CUDA(h, cudaFuncSetAttribute(k_ptc_corr, cudaFuncAttributeMaxDynamicSharedMemorySize, CORR_SMEM));
+        attr = true;
     }
-    std::vector<double> hd(4 * n + 4);
-    WD_CUDA(h, cudaMemcpyAsync(hd.data(), dots, sizeof(double) * (4 * n + 4), cudaMemcpyDeviceToHost, s));
-    WD_CUDA(h, cudaStreamSynchronize(s));
-    const int gx = grid_for(g.Vh, 128);
-    k_ptc_adjoint_weights<<<1, 256, 0, s>>>(B.weff + 2 * PTC_LAYER, B.wadj);
-    for (int i = 0; i < n; ++i) {
-        const float* vi = v + i * nf;
-        const float* yi = y + i * nf;
-        const double nv = hd[4 * i], ny = hd[4 * i + 1];
-        // forward: m = M v (hidden H kept for the weight gradient of layer 2)
-        WD_CUDA(h, ptc_apply_raw(h, WD_FP32, (const uint4*)vi, (uint4*)m, H, B.weff, le, lo, s, nullptr));
-        // e1 = m - y ; e2 = A m - v ; A^+ e2 = g5 A g5 e2
-        k_f32_lincomb<<<gv1, blk, 0, s>>>(nf, 1.f, m, -1.f, yi, e1);
-        WD_CUDA(h, apply_A_f32(h, (const uint4*)m, (uint4*)am, (uint4*)t1, le, lo, s));
-        k_f32_lincomb<<<gv1, blk, 0, s>>>(nf, 1.f, am, -1.f, vi, am);
-        dot(e1, e1, dots + 4 * i + 2);
-        dot(am, am, dots + 4 * i + 3);
-        k_gamma5_f32<<<gx, 128, 0, s>>>(g.Vh, (const uint4*)am, (uint4*)t2);
-        WD_CUDA(h, apply_A_f32(h, (const uint4*)t2, (uint4*)gv, (uint4*)t1, le, lo, s));
-        k_gamma5_f32<<<gx, 128, 0, s>>>(g.Vh, (const uint4*)gv, (uint4*)t2);
-        // g = 2 e1 / |y|^2 + 2 mu A^+ e2 / |v|^2  (= 2 dL/dconj(m))
-        k_f32_lincomb<<<gv1, blk, 0, s>>>(nf, (float)(2.0 / ny), e1, (float)(2.0 * mu / nv), t2, gv);
-        // layer 2: dW2 += sum g (x) conj(T_k H_c) ; g_H = adjoint network of layer 2 applied to g
-        k_ptc_wgrad<float, 18><<<wgrid, 128, 0, s>>>(g, 0, (const uint4*)gv, H, hvs, le, lo, wpart);
-        k_ptc_wgrad_sum<<<9 * PTC_C, 32, 0, s>>>(wgrid.x, wpart, B.grad + 2 * PTC_LAYER);
-        WD_CUDA(h, ptc_fanout_f32(h, (const uint4*)gv, GH, hvs, le, lo, B.wadj, s, err));
-        // layer 1: dW1 += sum g_H,c (x) conj(T_k v)
-        k_ptc_wgrad<float, 18><<<wgrid, 128, 0, s>>>(g, 1, GH, (const uint4*)vi, hvs, le, lo, wpart);
-        k_ptc_wgrad_sum<<<9 * PTC_C, 32, 0, s>>>(wgrid.x, wpart, B.grad);
+    for (int i0 = 0; i0 < n; i0 += chunk) {
+        const int nb = std::min(chunk, n - i0);
+        const uint4* vi = reinterpret_cast<const uint4*>(v) + i0 * vs;
+        const uint4* yi = reinterpret_cast<const uint4*>(y) + i0 * vs;
+        // m = M v ; e2 = A m - v ; b = A gamma5 e2 ; g = 2 (m - y) / |y|^2 + 2 mu gamma5 b / |v|^2
+        WD_CUDA(h, ptc_apply_f32(h, nb, vi, m, phi, B.V, le, lo, s));
+        WD_CUDA(h, apply_A_f32(h, nb, m, am, t1, le, lo, s));
+        k_ptc_resid<<<dim3(rb, nb), 256, 0, s>>>(g.Vh, vs, (const float4*)vi, (const float4*)yi, (const float4*)m,
+                                                 (const float4*)am, (float4*)t2, dpart);
+        k_ptc_dots<<<nb, 32, 0, s>>>(rb, dpart, dots + 4 * i0);
+        WD_CUDA(h, apply_A_f32(h, nb, t2, am, t1, le, lo, s));
+        k_ptc_lossgrad<<<dim3(gb, nb), 128, 0, s>>>(g.Vh, vs, vi, yi, m, am, dots + 4 * i0, mu, gv, c0part);
+        k_ptc_corr_sum<<<1, 256, 0, s>>>(gb * nb, 32, c0part, i0 > 0, C + CORR_FLOATS);
+        const int blocks = (int)std::min<long long>((long long)nb * ((g.Vh + CORR_SITES - 1) / CORR_SITES), cb);
+        k_ptc_corr<<<blocks, 128, CORR_SMEM, s>>>(g, nb, vi, gv, vs, lo, cpart);
+        k_ptc_corr_sum<<<CORR_FLOATS / 32, 256, 0, s>>>(blocks, CORR_FLOATS, cpart, i0 > 0, C);
         WD_CUDA(h, cudaGetLastError());
     }
-    WD_CUDA(h, cudaMemcpyAsync(hd.data(), dots, sizeof(double) * (4 * n + 4), cudaMemcpyDeviceToHost, s));
-    int herr = 0;
-    WD_CUDA(h, cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    k_ptc_wgrad<<<(2 * PTC_LAYER + 127) / 128, 128, 0, s>>>((const float2*)C, (const float2*)(C + CORR_FLOATS),
+                                                            (const float2*)B.weff, (float2*)B.grad);
+    WD_CUDA(h, cudaGetLastError());
+    std::vector<double> hd(4 * (size_t)n);
+    WD_CUDA(h, cudaMemcpyAsync(hd.data(), dots, sizeof(double) * hd.size(), cudaMemcpyDeviceToHost, s));
     WD_CUDA(h, cudaStreamSynchronize(s));
-    if (herr) return fail(h, WD_ERR_TIMEOUT, "wd_precond_grad: a bounded tensor-core wait gave up");
     double L = 0.0;
     for (int i = 0; i < n; ++i) L += hd[4 * i + 2] / hd[4 * i + 1] + mu * hd[4 * i + 3] / hd[4 * i];
     if (loss) *loss = L;
