@@ -160,17 +160,26 @@ class WDError(RuntimeError):
         self.code = code
 
 
+_current_raw_stream = None
+
+
 def _stream(stream):
+    """cudaStream_t of a stream (None: torch's current one) as an integer. The current stream is asked for on every
+    call, by its handle alone: building a torch.cuda.Stream object took 3.2 of the 9.3 us of a small wd_apply."""
+    global _current_raw_stream
     if stream is None:
-        import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if _current_raw_stream is None:
+            import torch
+            device, raw = torch.cuda.current_device, torch._C._cuda_getCurrentRawStream
+            _current_raw_stream = lambda: raw(device())  # noqa: E731
+        return _current_raw_stream()
     if isinstance(stream, int):
-        return C.c_void_p(stream)
-    return C.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def default_params(scheme) -> SolveParams:
