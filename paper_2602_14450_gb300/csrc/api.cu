@@ -451,8 +451,10 @@ static int apply_n(wd_handle* h, int prec, int recon, int op, int nrhs, const vo
                                 op == WD_OP_EO_A ? &ci_o : &cf_o)) != WD_OK)
             return rc;
     }
+    int nth = 0;   // the hops of an operator sweep the sites up and down in turn
     auto hop = [&](int parity, const void* src, void* dst, int epi, double a, double b, const void* y,
                    const uint4* mat = nullptr) {
+        P.rev = nth++ & 1;
         P.mat = mat;
         P.parity = parity;
         P.links = parity == 0 ? le : lo;

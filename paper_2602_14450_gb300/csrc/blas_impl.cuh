@@ -54,13 +54,15 @@ __device__ __forceinline__ void store_unit(uint4* v, size_t off, typename Unit<T
     for (int i = 0; i < Unit<T>::N; ++i) c[i] = Unit<T>::get(w, i);
 }
 
-// Per right-hand-side loop over groups of S sites of a batched launch: sites h, h + step, ... h + (S-1) step.
-#define RHS_LOOP_S(h, n, S) for (int h = sl.b * blockDim.x + threadIdx.x; h < (n); h += (S) * sl.nb * blockDim.x)
+// Per right-hand-side loop over groups of S sites of a batched launch, counted in sweep order: a block takes S
+// blockDim.x consecutive ones, its threads i, i + step, ... i + (S-1) step with step = blockDim.x.
+#define RHS_LOOP_S(i, n, S) \
+    for (int i = (S) * sl.b * blockDim.x + threadIdx.x; i < sweep_end(n); i += (S) * sl.nb * blockDim.x)
 
 // p := r (first iteration) or cP p - cV v + r
 template <typename T>
 __global__ void __launch_bounds__(256) k_pupdate(int n, int nrhs, long long vs, uint4* p, const uint4* v,
-                                                 const uint4* r, const SolverState* sts) {
+                                                 const uint4* r, const SolverState* sts, int rev) {
     pdl_begin();
     typedef typename Unit<T>::C C;
     typedef Stream<T> ST;
@@ -71,15 +73,15 @@ __global__ void __launch_bounds__(256) k_pupdate(int n, int nrhs, long long vs, 
     p += ro; v += ro; r += ro;
     const bool first = st->first, ftz = st->ftz;
     const C pr = (C)st->cP[0], pi = (C)st->cP[1], vr = (C)st->cV[0], vi = (C)st->cV[1];
-    const int step = sl.nb * blockDim.x;
-    RHS_LOOP_S(h0, n, ST::SITES) {
+    const int step = blockDim.x;
+    RHS_LOOP_S(i0, n, ST::SITES) {
 #pragma unroll
         for (int u0 = 0; u0 < ST::SU; u0 += ST::CH) {
             uint4 ur[ST::SITES][ST::CH], up[ST::SITES][ST::CH], uv[ST::SITES][ST::CH];
 #pragma unroll
             for (int q = 0; q < ST::SITES; ++q) {
-                const int h = h0 + q * step;
-                if (h >= n) continue;
+                const int h = sweep_site(i0 + q * step, n, rev);
+                if ((unsigned)h >= (unsigned)n) continue;
 #pragma unroll
                 for (int c = 0; c < ST::CH; ++c) {
                     const size_t off = (size_t)(u0 + c) * n + h;
@@ -92,8 +94,8 @@ __global__ void __launch_bounds__(256) k_pupdate(int n, int nrhs, long long vs, 
             }
 #pragma unroll
             for (int q = 0; q < ST::SITES; ++q) {
-                const int h = h0 + q * step;
-                if (h >= n) continue;
+                const int h = sweep_site(i0 + q * step, n, rev);
+                if ((unsigned)h >= (unsigned)n) continue;
 #pragma unroll
                 for (int c = 0; c < ST::CH; ++c) {
                     C o[ST::N];
@@ -118,7 +120,7 @@ __global__ void __launch_bounds__(256) k_pupdate(int n, int nrhs, long long vs, 
 // r := r - alpha v
 template <typename T>
 __global__ void __launch_bounds__(256) k_supdate(int n, int nrhs, long long vs, uint4* r, const uint4* v,
-                                                 const SolverState* sts) {
+                                                 const SolverState* sts, int rev) {
     pdl_begin();
     typedef typename Unit<T>::C C;
     typedef Stream<T> ST;
@@ -129,15 +131,15 @@ __global__ void __launch_bounds__(256) k_supdate(int n, int nrhs, long long vs, 
     r += o; v += o;
     const bool ftz = st->ftz;
     const C ar = (C)-st->alpha[0], ai = (C)-st->alpha[1];
-    const int step = sl.nb * blockDim.x;
-    RHS_LOOP_S(h0, n, ST::SITES) {
+    const int step = blockDim.x;
+    RHS_LOOP_S(i0, n, ST::SITES) {
 #pragma unroll
         for (int u0 = 0; u0 < ST::SU; u0 += ST::CH) {
             uint4 ur[ST::SITES][ST::CH], uv[ST::SITES][ST::CH];
 #pragma unroll
             for (int q = 0; q < ST::SITES; ++q) {
-                const int h = h0 + q * step;
-                if (h >= n) continue;
+                const int h = sweep_site(i0 + q * step, n, rev);
+                if ((unsigned)h >= (unsigned)n) continue;
 #pragma unroll
                 for (int c = 0; c < ST::CH; ++c) {
                     const size_t off = (size_t)(u0 + c) * n + h;
@@ -147,8 +149,8 @@ __global__ void __launch_bounds__(256) k_supdate(int n, int nrhs, long long vs, 
             }
 #pragma unroll
             for (int q = 0; q < ST::SITES; ++q) {
-                const int h = h0 + q * step;
-                if (h >= n) continue;
+                const int h = sweep_site(i0 + q * step, n, rev);
+                if ((unsigned)h >= (unsigned)n) continue;
 #pragma unroll
                 for (int c = 0; c < ST::CH; ++c) {
                     C rr[ST::N];
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(256) k_supdate(int n, int nrhs, long long vs, 
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) k_xr(int n, int nrhs, long long vs, uint4* x, uint4* r, const uint4* p,
                                             const uint4* t, const uint4* rstar, const uint4* xr_src,
-                                            const uint4* xp_src, SolverState* sts, RedCtx rc) {
+                                            const uint4* xp_src, SolverState* sts, RedCtx rc, int rev) {
     pdl_begin();
     typedef typename Unit<T>::C C;
     typedef Stream<T> ST;
@@ -193,7 +195,9 @@ __global__ void __launch_bounds__(256) k_xr(int n, int nrhs, long long vs, uint4
     const C om_r = (C)-st->omega[0], om_i = (C)-st->omega[1];
     const C gs = MODE == XR_FUSED ? (C)st->gam_tmp : (C)1;
     C s_r2 = 0, s_x2 = 0, s_re = 0, s_im = 0;
-    RHS_LOOP(h, n) {
+    RHS_LOOP_S(i, n, 1) {
+        const int h = sweep_site(i, n, rev);
+        if (h >= n) continue;
 #pragma unroll
         for (int u0 = 0; u0 < ST::SU; u0 += ST::CH) {
             uint4 ur[ST::CH], up[ST::CH], ux[ST::CH], ut[ST::CH], urs[ST::CH], urr[ST::CH];

@@ -682,6 +682,15 @@ __device__ __forceinline__ Slice slice_of(int nrhs) {
     return s;
 }
 
+// Order of the sites of a launch. Blocks start in the order of their index, so
+// a kernel that takes the sites downwards begins where one that took them
+// upwards ended, with what that kernel wrote and read last still in the L2
+// (129 MB). The kernels of a chain over vectors that do not fit there alternate.
+// i counts a launch's sites upwards; the order is turned warp by warp, which
+// keeps each warp's 32 sites together. Sites at or beyond n are skipped.
+__device__ __forceinline__ int sweep_end(int n) { return (n + 31) & ~31; }
+__device__ __forceinline__ int sweep_site(int i, int n, int rev) { return rev ? (sweep_end(n) - 32 - (i & ~31)) | (i & 31) : i; }
+
 // Sums of FP64 values. The FP64 pipe takes 64 cycles per warp instruction (half a lane per cycle and SM
 // sub-partition), so the sums are folded instead of reduced one after the other: exchanging with the lane 16
 // away, a lane keeps half of the sums, then with the lane 8 away a quarter, and the last steps add one value per

@@ -291,7 +291,9 @@ __global__ void __launch_bounds__(Hop16Bounds<R, RED, MAT, AHEAD>::THREADS, Hop1
 #pragma unroll
     for (int k = 0; k < NS; ++k) part[k] = 0.f;
 
-    for (int h = sl.b * blockDim.x + threadIdx.x; h < Vh; h += sl.nb * blockDim.x) {
+    for (int i = sl.b * blockDim.x + threadIdx.x; i < sweep_end(Vh); i += sl.nb * blockDim.x) {
+        const int h = sweep_site(i, Vh, P.rev);
+        if (h >= Vh) continue;
         int nbr[8];
         const unsigned wm = site_neighbours(g, P.parity, h, nbr);
         __half2 acc[12];

@@ -56,6 +56,7 @@ struct HopParams {
     int rhs_group[2];          // FP16 arithmetic: right-hand sides per thread (hop16m_kernel) without / with a
                                // fused reduction; 0 or 1 = one (hop16_kernel); must divide nrhs to be used
     int rhs_smem[2];           // ... and 1 = the site's links in shared memory instead of registers
+    int rev;                   // 1 = take the sites from the last to the first (sweep_site; FP16 arithmetic)
     int fixed64;               // FP64, 18-real: the links are fixed-point digits (hop64_kernel)
     int spt;                   // FP16 arithmetic, plain hop: sites per thread (grid-stride; 0 or 1 = one site)
 };
@@ -74,14 +75,15 @@ int spinor_units(int prec);
 // (vs64 for FP64 vectors), st = state array, g = guard kind.
 template <typename T> struct Ops {
     static cudaError_t hop(int recon, int epi, int red, const HopParams& P, cudaStream_t s);
+    // rev: order of the sites (sweep_site)
     static cudaError_t pupdate(int n, int nrhs, long long vs, uint4* p, const uint4* v, const uint4* r,
-                               const SolverState* st, cudaStream_t s);
+                               const SolverState* st, int rev, cudaStream_t s);
     static cudaError_t supdate(int n, int nrhs, long long vs, uint4* r, const uint4* v, const SolverState* st,
-                               cudaStream_t s);
+                               int rev, cudaStream_t s);
     // mode: XrMode
     static cudaError_t xr(int mode, int n, int nrhs, long long vs, uint4* x, uint4* r, const uint4* p,
                           const uint4* t, const uint4* rstar, const uint4* xr_src, const uint4* xp_src,
-                          SolverState* st, RedCtx rc, cudaStream_t s);
+                          SolverState* st, RedCtx rc, int rev, cudaStream_t s);
     static cudaError_t scale(int n, int nrhs, long long vs, uint4* r, uint4* x, const uint4* rstar, SolverState* st,
                              RedCtx rc, cudaStream_t s);
     static cudaError_t rescale_in(int n, int nrhs, long long vs, long long vs64, const uint4* r64, uint4* r,

@@ -92,6 +92,7 @@ extern "C" int wd_apply_eo_noalloc(wd_handle* h, int prec, int recon, const void
     const double k = h->kappa;
     auto hop = [&](int parity, const void* src, void* dst, int epi, double a, double b, const void* y,
                    const uint4* mat) {
+        P.rev = parity == 0 ? 1 : 0;   // the second hop sweeps the sites downwards, as in wd_apply
         P.mat = mat;
         P.parity = parity;
         P.links = parity == 0 ? le : lo;

@@ -292,28 +292,28 @@ cudaError_t Ops<T>::chiral_from64(int n, const uint4* src64, uint4* dst, cudaStr
 
 template <typename T>
 cudaError_t Ops<T>::pupdate(int n, int nrhs, long long vs, uint4* p, const uint4* v, const uint4* r,
-                            const SolverState* st, cudaStream_t s) {
+                            const SolverState* st, int rev, cudaStream_t s) {
     const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, VEC_BLOCK);
-    { const cudaError_t le_ = launch_k(k_pupdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, p, v, r, st); if (le_ != cudaSuccess) return le_; }
+    { const cudaError_t le_ = launch_k(k_pupdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, p, v, r, st, rev); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::supdate(int n, int nrhs, long long vs, uint4* r, const uint4* v, const SolverState* st,
-                            cudaStream_t s) {
+                            int rev, cudaStream_t s) {
     const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, VEC_BLOCK);
-    { const cudaError_t le_ = launch_k(k_supdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, r, v, st); if (le_ != cudaSuccess) return le_; }
+    { const cudaError_t le_ = launch_k(k_supdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, r, v, st, rev); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Ops<T>::xr(int mode, int n, int nrhs, long long vs, uint4* x, uint4* r, const uint4* p,
                        const uint4* t, const uint4* rstar, const uint4* xr_src, const uint4* xp_src,
-                       SolverState* st, RedCtx rc, cudaStream_t s) {
+                       SolverState* st, RedCtx rc, int rev, cudaStream_t s) {
 #define WD_XR_CASE(M)                                                                                        \
     if (mode == M) {                                                                                         \
         const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_xr<T, M>, n, block, nrhs);                            \
-        { const cudaError_t le_ = launch_k(k_xr<T, M>, nb * nrhs, block, 0, s, n, nrhs, vs, x, r, p, t, rstar, xr_src, xp_src, st, rc); if (le_ != cudaSuccess) return le_; }   \
+        { const cudaError_t le_ = launch_k(k_xr<T, M>, nb * nrhs, block, 0, s, n, nrhs, vs, x, r, p, t, rstar, xr_src, xp_src, st, rc, rev); if (le_ != cudaSuccess) return le_; }   \
         return cudaGetLastError();                                                                           \
     }
     WD_XR_CASE(XR_PLAIN)

@@ -173,13 +173,16 @@ static cudaError_t hop64(const Sys& S, int parity, const uint4* in, uint4* out, 
 // Enqueue one inner BiCGStab iteration (Alg. 4 / Alg. 5 loop body) of every
 // right-hand side of a system; with a right preconditioner M the operator is
 // A M: v = A (M p), t = A (M s), x += lambda'/gamma' (omega M s + alpha M p).
-static cudaError_t enqueue_iteration(const Sys& S, int prec, int recon, int xr_mode, bool learned,
+// The kernels sweep the sites up and down in turn (sweep_site), carried on from iteration to iteration: `it`.
+static cudaError_t enqueue_iteration(const Sys& S, int prec, int recon, int xr_mode, bool learned, int it,
                                      cudaStream_t s) {
     const int n = S.h->g.Vh, nr = S.nrhs;
     const long long vs = S.vs;
     const double k2 = S.h->kappa * S.h->kappa;
     SolverState* st = S.h->st;
     wd_handle* h = S.h;
+    int up = it & 1;   // seven alternating kernels an iteration
+    const auto turn = [&up]() { return (up ^= 1) ^ 1; };
     return by_prec(prec, [&](auto tag) -> cudaError_t {
         typedef typename decltype(tag)::type T;
         cudaError_t e;
@@ -187,7 +190,7 @@ static cudaError_t enqueue_iteration(const Sys& S, int prec, int recon, int xr_m
         apply_tuning(h, prec, recon, P);
         P.vs = vs;
         // p := beta (p - omega' v) + r   (gamma of p and v folded in)
-        if ((e = Ops<T>::pupdate(n, nr, vs, S.p, S.v, S.r, st, s)) != cudaSuccess) return e;
+        if ((e = Ops<T>::pupdate(n, nr, vs, S.p, S.v, S.r, st, turn(), s)) != cudaSuccess) return e;
         const uint4* pa = S.p;   // operand of A
         if (learned) {
             if ((e = ptc_apply_m(h, WD_FP16, S.p, S.phat, S.PHI, S.V, S.le, S.lo, s, st, S.err)) != cudaSuccess) return e;
@@ -195,12 +198,14 @@ static cudaError_t enqueue_iteration(const Sys& S, int prec, int recon, int xr_m
         }
         // v = A p = p - kappa^2 H_eo H_oe p ; alpha = rho / (r*, v)
         P.parity = 1; P.links = S.lo; P.in = pa; P.out = S.tmp; P.a = 1.0; P.mat = S.mio;
+        P.rev = turn();
         if ((e = Ops<T>::hop(recon, EPI_H, RED_NONE, P, s)) != cudaSuccess) return e;
         P.parity = 0; P.links = S.le; P.in = S.tmp; P.out = S.v; P.y = pa; P.a = -k2; P.b = 1.0; P.mat = S.mie;
         P.rstar = S.rs; P.rc = red_ctx(h, ST_ALPHA);
+        P.rev = turn();
         if ((e = Ops<T>::hop(recon, EPI_Y, RED_RSV, P, s)) != cudaSuccess) return e;
         // r := r - alpha v
-        if ((e = Ops<T>::supdate(n, nr, vs, S.r, S.v, st, s)) != cudaSuccess) return e;
+        if ((e = Ops<T>::supdate(n, nr, vs, S.r, S.v, st, turn(), s)) != cudaSuccess) return e;
         const uint4* sa = S.r;   // operand of A
         if (learned) {
             if ((e = ptc_apply_m(h, WD_FP16, S.r, S.shat, S.PHI, S.V, S.le, S.lo, s, st, S.err)) != cudaSuccess) return e;
@@ -210,16 +215,18 @@ static cudaError_t enqueue_iteration(const Sys& S, int prec, int recon, int xr_m
         P.rc = red_ctx(h, ST_NONE);
         P.parity = 1; P.links = S.lo; P.in = sa; P.out = S.tmp; P.y = nullptr; P.a = 1.0; P.b = 0.0;
         P.rstar = nullptr; P.mat = S.mio;
+        P.rev = turn();
         if ((e = Ops<T>::hop(recon, EPI_H, RED_NONE, P, s)) != cudaSuccess) return e;
         P.parity = 0; P.links = S.le; P.in = S.tmp; P.out = S.t; P.y = sa; P.a = -k2; P.b = 1.0; P.mat = S.mie;
         P.rstar = learned ? S.r : nullptr;   // dot partner s when t = A M s
         P.rc = red_ctx(h, ST_OMEGA);
+        P.rev = turn();
         if ((e = Ops<T>::hop(recon, EPI_Y, RED_TS, P, s)) != cudaSuccess) return e;
         // x += lambda'/gamma' (omega s + alpha p) ; r := s - omega t ; |r|, |x|
         //   (with XR_FUSED r is stored rescaled and the iteration ends here)
         if ((e = Ops<T>::xr(xr_mode, n, nr, vs, S.xt, S.r, S.p, S.t, S.rs, learned ? S.shat : nullptr,
                             learned ? S.phat : nullptr, st, red_ctx(h, xr_mode == XR_FUSED ? ST_RFUSED : ST_RNORM),
-                            s)) != cudaSuccess)
+                            turn(), s)) != cudaSuccess)
             return e;
         // r := (sigma / g) r ; gamma ; [x := lambda x] ; next rho, beta
         if (xr_mode == XR_NORMS)
@@ -249,7 +256,7 @@ static int capture_inner(std::vector<Sys>& sys, int prec, int recon, int xr_mode
         for (size_t i = 1; i < sys.size() && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(sys[i].h->cap, h0->ev[1], 0);
         for (size_t i = 0; i < sys.size() && e == cudaSuccess; ++i)
             for (int it = 0; it < iters && e == cudaSuccess; ++it)
-                e = enqueue_iteration(sys[i], prec, recon, xr_mode, learned, sys[i].h->cap);
+                e = enqueue_iteration(sys[i], prec, recon, xr_mode, learned, it, sys[i].h->cap);
         for (size_t i = 1; i < sys.size() && e == cudaSuccess; ++i) {              // join
             e = cudaEventRecord(sys[i].h->ev[0], sys[i].h->cap);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(h0->cap, sys[i].h->ev[0], 0);
@@ -257,7 +264,7 @@ static int capture_inner(std::vector<Sys>& sys, int prec, int recon, int xr_mode
     } else {
         for (int i = 0; i < iters && e == cudaSuccess; ++i)
             for (auto& S : sys)
-                if (e == cudaSuccess) e = enqueue_iteration(S, prec, recon, xr_mode, learned, h0->cap);
+                if (e == cudaSuccess) e = enqueue_iteration(S, prec, recon, xr_mode, learned, i, h0->cap);
     }
     for (size_t i = 0; i < sys.size() && e == cudaSuccess; ++i) {   // the activity flag, in mapped host memory
         k_any_active<<<1, 1024, 0, h0->cap>>>(sys[i].nrhs, sys[i].h->st, h0->dflag, i > 0 ? 1 : 0);
