@@ -94,6 +94,18 @@ void* workspace(wd_handle* h, const std::string& name, size_t bytes) {
     return b.p;
 }
 
+int* lower_err(wd_handle* h) {
+    if (!h->herr) {
+        if (cudaHostAlloc((void**)&h->herr, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+            h->herr = nullptr;
+            return nullptr;
+        }
+        if (cudaHostGetDevicePointer((void**)&h->derr, h->herr, 0) != cudaSuccess) return nullptr;
+    }
+    *(volatile int*)h->herr = 0;
+    return h->derr;
+}
+
 RedCtx red_ctx(wd_handle* h, int stage) {
     RedCtx rc;
     rc.partials = h->partials;
@@ -307,6 +319,7 @@ int wd_destroy(wd_handle* h) {
     if (h->ticket) cudaFree(h->ticket);
     if (h->hst) cudaFreeHost(h->hst);
     if (h->hflag) cudaFreeHost(h->hflag);
+    if (h->herr) cudaFreeHost(h->herr);
     if (h->cap) cudaStreamDestroy(h->cap);
     for (int i = 0; i < 2; ++i)
         if (h->ev[i]) cudaEventDestroy(h->ev[i]);

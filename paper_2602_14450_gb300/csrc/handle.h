@@ -75,6 +75,8 @@ struct wd_handle {
 
     int arith16 = 0;                   // wd_set_arith: FP16-storage hops sum in FP16 arithmetic
 
+    int* herr = nullptr;               // mapped pinned host word: raised by a kernel whose bounded wait gave up, read
+    int* derr = nullptr;               // after the call's synchronisation; its device address
     unsigned wait_rounds = 0;          // wd_set_wait_limit: rounds of a bounded device wait + 1; 0 = the default
 
     int dd_grid[4] = {1, 1, 1, 1};     // wd_dd_set_partition: processes per direction
@@ -92,6 +94,9 @@ int ensure_solver_state(wd_handle* h, int nrhs);
 int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const uint4** odd);
 size_t vec_bytes(const wd_handle* h, int prec);
 RedCtx red_ctx(wd_handle* h, int stage);
+// Device address of the handle's timeout flag, lowered; null on failure. Calls that may raise it read it from
+// h->herr once their stream has been synchronised.
+int* lower_err(wd_handle* h);
 // Clover blocks (clover.cu): rebuild from the gauge field; fetch kind 0 (C^-1)
 // or 1 (C) in a precision (null pointers without a clover term).
 int clover_build(wd_handle* h);

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(128) hop3_kernel(const HopParams P, const Stag
         }
         const bool landed = mbar_wait(&bar, phase, P.wait_rounds ? P.wait_rounds - 1 : MBAR_WAIT_LIMIT);
         if (__syncthreads_or(!landed)) {              // uniform across the block
-            if (threadIdx.x == 0 && err) atomicExch(err, 1);
+            if (threadIdx.x == 0 && err) *(volatile int*)err = 1;
             mbar_wait(&bar, phase);                   // default bound: let the copies land before the block goes on
             break;                                    // still takes its part in the grid reduction below
         }

@@ -616,8 +616,6 @@ static int ptc_bufs(wd_handle* h, PtcBufs* b) {
     return WD_OK;
 }
 
-int* ptc_err(wd_handle* h);
-
 // Whether the first pass of the FP16 path of M mixes channels on the tensor
 // cores (environment WD_PTC_TC=0 selects the FP32-core kernel).
 static bool ptc_tensor_cores() {
@@ -628,9 +626,6 @@ static bool ptc_tensor_cores() {
     }
     return v == 1;
 }
-
-// Device flag raised by a kernel whose bounded wait gave up.
-int* ptc_err(wd_handle* h) { return (int*)workspace(h, "ptc.err", sizeof(int)); }
 
 // Intermediate fields phi_{1+d} of the collapsed M: 8 odd-site vectors in the
 // storage type of `prec` (FP32 for WD_FP32, BF16 otherwise).
@@ -822,15 +817,12 @@ extern "C" int wd_precond_apply(wd_handle* h, int prec, const void* in, void* ou
     const uint4 *le, *lo;
     if ((rc = ensure_links(h, prec, prec == WD_FP32 ? 18 : 12, &le, &lo)) != WD_OK) return rc;
     uint4* PHI = ptc_phi(h, prec);
-    int* err = ptc_err(h);
+    int* err = lower_err(h);
     if (!PHI || !err) return fail(h, WD_ERR_CUDA, "out of device memory");
     cudaStream_t s = (cudaStream_t)stream;
-    WD_CUDA(h, cudaMemsetAsync(err, 0, sizeof(int), s));
     WD_CUDA(h, ptc_apply_m(h, prec, (const uint4*)in, (uint4*)out, PHI, B.V, le, lo, s, nullptr, err));
-    int herr = 0;
-    WD_CUDA(h, cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     WD_CUDA(h, cudaStreamSynchronize(s));
-    if (herr) return fail(h, WD_ERR_TIMEOUT, "wd_precond_apply: a bounded tensor-core wait gave up");
+    if (*(volatile int*)h->herr) return fail(h, WD_ERR_TIMEOUT, "wd_precond_apply: a bounded tensor-core wait gave up");
     return WD_OK;
 }
 

@@ -31,7 +31,6 @@ struct SchemeCfg {
 
 cudaError_t ptc_apply_m(wd_handle* h, int prec, const uint4* in_e, uint4* out_e, uint4* PHI, const float2* V,
                         const uint4* le, const uint4* lo, cudaStream_t s, const SolverState* guard, int* err);
-int* ptc_err(wd_handle* h);
 const float2* ptc_collapsed(wd_handle* h);
 uint4* ptc_phi16(wd_handle* h);
 
@@ -113,9 +112,8 @@ static int prepare(Sys& S, int prec, int recon_lo, bool learned) {
         if (!*flo[i]) return fail(h, WD_ERR_CUDA, "out of device memory (%s)", nlo[i]);
     }
     // raised by any kernel of the solve whose bounded device wait gave up
-    S.err = ptc_err(h);
-    if (!S.err) return fail(h, WD_ERR_CUDA, "out of device memory");
-    if (cudaMemset(S.err, 0, sizeof(int)) != cudaSuccess) return fail(h, WD_ERR_CUDA, "cudaMemset");
+    S.err = lower_err(h);
+    if (!S.err) return fail(h, WD_ERR_CUDA, "out of pinned host memory");
     if (learned) {
         S.phat = (uint4*)workspace(h, pre + "phat", blo);
         S.shat = (uint4*)workspace(h, pre + "shat", blo);
@@ -595,12 +593,7 @@ int solve_systems(int n, wd_handle* const* hs, const int* nrhs, const double* co
     WD_CUDA(h0, cudaEventRecord(h0->t1, s));
     if ((rc = read_states(sys, s)) != WD_OK) return rc;
     bool timed_out = false;   // a bounded device wait of a kernel gave up
-    for (auto& S : sys) {
-        if (!S.err) continue;
-        int herr = 0;
-        WD_CUDA(S.h, cudaMemcpy(&herr, S.err, sizeof(int), cudaMemcpyDeviceToHost));
-        timed_out = timed_out || herr != 0;
-    }
+    for (auto& S : sys) timed_out = timed_out || *(volatile int*)S.h->herr != 0;
     float ms = 0;
     cudaEventElapsedTime(&ms, h0->t0, h0->t1);
     int worst = WD_OK;
