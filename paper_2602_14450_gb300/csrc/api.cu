@@ -11,23 +11,21 @@
 
 namespace wd {
 
-static int g_hop_block = 0;
-// Default threads per block of the hop kernels: environment WD_HOP_BLOCK (64 or 128), else 128.
 int hop_block() {
-    if (g_hop_block == 0) {
+    static int v = -1;
+    if (v < 0) {
         const char* e = std::getenv("WD_HOP_BLOCK");
         const int b = e ? std::atoi(e) : 0;
-        g_hop_block = (b == 64 || b == 128) ? b : 128;
+        v = (b == 64 || b == 128) ? b : 0;
     }
-    return g_hop_block;
+    return v;
 }
-void set_hop_block(int b) { g_hop_block = b; }
 
 int hop_variant() {
-    static int v = 0;
-    if (v == 0) {
+    static int v = -1;
+    if (v < 0) {
         const char* e = std::getenv("WD_HOP_KERNEL");
-        v = (e && e[0] >= '1' && e[0] <= '6') ? e[0] - '0' : 4;
+        v = (e && e[0] >= '1' && e[0] <= '6') ? e[0] - '0' : 0;
     }
     return v;
 }

@@ -109,20 +109,21 @@ template <typename T> struct Ops {
 
 cudaError_t launch_unitarity(int nlinks, const double* U, unsigned long long* out, cudaStream_t s);
 
-// Block size of every vector kernel; the hop kernels take theirs from
-// HopParams::block (set by wd_tune) or else hop_block() (environment
-// WD_HOP_BLOCK = 64 or 128, default 128).
+// Block size of every vector kernel. The hop kernels take theirs from
+// HopParams::block (set by wd_tune), else from the environment (WD_HOP_BLOCK =
+// 64 or 128), else by rule (default_block).
 constexpr int VEC_BLOCK = 256;
-int hop_block();
-void set_hop_block(int b);
-// Hop kernel variant, read once from the environment variable WD_HOP_KERNEL:
+int hop_block();     // the environment's, 0 = none
+// Hop kernel variant, from HopParams::variant, else from the environment
+// (WD_HOP_KERNEL), else by rule (default_variant):
 // 4 = one site per thread, neighbour and link loads issued one direction
-// ahead (default); 1 = one site per thread without the look-ahead; for
-// FP32-arithmetic storage 2 = two sites per thread with packed FP32x2 math;
-// for 16-bit storage 3 = tiles staged in shared memory by bulk copies and,
-// with 12-real links, 5 = persistent threads streaming their operands through
-// a per-thread two-slot ring of asynchronous copies in shared memory.
-int hop_variant();
+// ahead; 1 = one site per thread without the look-ahead; 6 = as 4 with the
+// SU(3) products on FP32x2 pairs; for FP32-arithmetic storage 2 = two sites per
+// thread with packed FP32x2 math; for 16-bit storage 3 = tiles staged in shared
+// memory by bulk copies and, with 12-real links, 5 = persistent threads
+// streaming their operands through a per-thread two-slot ring of asynchronous
+// copies in shared memory.
+int hop_variant();   // the environment's, 0 = none
 // Directions ahead that the FP16-arithmetic hop loads its neighbour spinors
 // (environment WD_HOP16_AHEAD = 1 or 2, default 2: 3% faster at 32^3 x 64).
 int hop16_ahead();

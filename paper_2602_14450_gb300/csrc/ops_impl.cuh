@@ -84,6 +84,27 @@ inline int spread_block(int n, int nrhs, int block) {
     return block;
 }
 
+// Hop kernel variant and block size of a lattice without wd_tune's choice, from
+// the plain hop (us, GB300) at Vh = 65536 | 120960 | 160000 | 331776 | 1048576:
+//   BF16, 18-real   4: 9.41 11.5 13.1 22.7 70.2   1: 6.61 10.1 12.8 22.5 71.4   6: 8.35 12.1 13.3 22.0 72.0
+//   BF16, 12-real   4: 8.92 11.3 13.3 23.0 67.1   1: 6.74 10.6 13.1 23.5 70.4   6: 8.16 11.1 12.7 21.6 65.0
+//   FP16, 18-real   4: 7.00 10.1 12.7 20.7 65.8   1: 6.39 9.84 12.4 21.6 69.7
+// Over few sites the 16-bit look-ahead kernels, held to 80 registers for the
+// occupancy of a large lattice, lose more to spills than the loads ahead give;
+// the kernel without look-ahead takes 128. With a clover block (even-odd
+// operator, two hops): FP16 21.4 26.3 - 58.0 against 16.0 24.7 - 61.7 without
+// look-ahead, BF16 22.5 28.0 - 62.5 against 14.9 23.3 - 63.2 (on FP32x2 pairs).
+// FP32 storage and the clover hops run 1-2% faster in blocks of 64 threads.
+constexpr int FEW_SITES = 160000;
+template <typename T, int R> int default_variant(const Geom& g) {
+    if (std::is_same<T, __nv_bfloat16>::value) return g.Vh <= FEW_SITES ? 1 : R == 12 ? 6 : 4;
+    if (std::is_same<T, __half>::value && R == 18) return g.Vh <= FEW_SITES ? 1 : 4;
+    return 4;
+}
+template <typename T> constexpr int default_block(bool reducing) {
+    return std::is_same<T, float>::value && !reducing ? 64 : 128;
+}
+
 // Tiling of the staged hop kernel, or false when its shared memory would not
 // allow two resident blocks per SM.
 template <typename T, int R>
@@ -181,16 +202,22 @@ cudaError_t run_hop(const HopParams& P, cudaStream_t s) {
     if constexpr (std::is_same<T, double>::value && R == 18) {
         if (P.fixed64) return P.mat ? run_hop64<E, D, true>(P, s) : run_hop64<E, D, false>(P, s);
     }
-    if (P.mat) {   // with a site-local block (clover): the one-site-per-thread look-ahead kernel
-        const int blk = spread_block(P.g.Vh, P.nrhs, 128);
-        const void* km = (const void*)hop_kernel<T, R, E, D, true, false, true>;
-        const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, blk) : reduce_blocks(km, P.g.Vh, blk, P.nrhs);
-        { const cudaError_t le_ = launch_k(hop_kernel<T, R, E, D, true, false, true>, nb * P.nrhs, blk, 0, s, P); if (le_ != cudaSuccess) return le_; }
-        return cudaGetLastError();
+    if (P.mat) {   // with a site-local block (clover): one site per thread, with look-ahead but for 16 bits on few sites
+        const int blk = spread_block(P.g.Vh, P.nrhs, D == RED_NONE ? 64 : 128);
+        const auto run = [&](auto kernel) -> cudaError_t {
+            const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, blk)
+                                           : reduce_blocks((const void*)kernel, P.g.Vh, blk, P.nrhs);
+            const cudaError_t e = launch_k(kernel, nb * P.nrhs, blk, 0, s, P);
+            return e != cudaSuccess ? e : cudaGetLastError();
+        };
+        if constexpr (sizeof(T) == 2)
+            if (P.g.Vh <= FEW_SITES) return run(hop_kernel<T, R, E, D, false, std::is_same<T, __nv_bfloat16>::value, true>);
+        return run(hop_kernel<T, R, E, D, true, false, true>);
     }
     constexpr int form = D == RED_NONE ? 0 : 1;
-    const int block = spread_block(P.g.Vh, P.nrhs, P.block[form] > 0 ? P.block[form] : hop_block());
-    const int variant = P.variant[form] > 0 ? P.variant[form] : hop_variant();
+    const int block = spread_block(P.g.Vh, P.nrhs, P.block[form] > 0 ? P.block[form]
+                                                   : hop_block() ? hop_block() : default_block<T>(D != RED_NONE));
+    const int variant = P.variant[form] > 0 ? P.variant[form] : hop_variant() ? hop_variant() : default_variant<T, R>(P.g);
     const int nr = P.nrhs;
     if constexpr (sizeof(T) == 2) {
         StageGeom sg;
