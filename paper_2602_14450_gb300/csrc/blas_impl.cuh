@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256) k_supdate(int n, int nrhs, long long vs, 
 // x := x + cXr r + cXp p  (x := cXr r + cXp p on the first iteration)
 // r := r - omega t, and with XR_FUSED stored as c (r - omega t), c = sigma / g~
 // the rescaling factor from the predicted norm (ST_OMEGA)
-// sums: XR_PLAIN  |r|^2, |x|^2, (r*, r)
+// sums: XR_PLAIN  |r|^2, 0, (r*, r)     (|x|^2 serves the rescaling of x alone)
 //       XR_NORMS  |r|^2, |x|^2            (a separate k_scale pass follows)
 //       XR_FUSED  |r|^2 (before scaling), |r_stored|^2, (r*, r_stored)
 // One site per thread and step: six vectors of a site are in flight at once.
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(256) k_xr(int n, int nrhs, long long vs, uint4
                 if constexpr (MODE == XR_FUSED) {
 #pragma unroll
                     for (int i = 0; i < ST::N; ++i) s_x2 += rr[i] * rr[i];      // |r_stored|^2
-                } else {
+                } else if constexpr (MODE == XR_NORMS) {
 #pragma unroll
                     for (int i = 0; i < ST::N; ++i) s_x2 += xx[i] * xx[i];
                 }

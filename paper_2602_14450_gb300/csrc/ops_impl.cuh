@@ -84,6 +84,11 @@ inline int spread_block(int n, int nrhs, int block) {
     return block;
 }
 
+// Threads per block of the solver's vector kernels. In FP64 an SM works through its sites at the rate of its FP64
+// pipe, so small blocks share them out evenly: at 16^3 x 32, 256 blocks of 256 threads gave half of the SMs twice
+// the sites of the others.
+template <typename T> constexpr int vec_block() { return sizeof(T) == 8 ? 64 : VEC_BLOCK; }
+
 // Hop kernel variant and block size of a lattice without wd_tune's choice, from
 // the plain hop (us, GB300) at Vh = 65536 | 120960 | 160000 | 331776 | 1048576:
 //   BF16, 18-real   4: 9.41 11.5 13.1 22.7 70.2   1: 6.61 10.1 12.8 22.5 71.4   6: 8.35 12.1 13.3 22.0 72.0
@@ -320,7 +325,7 @@ cudaError_t Ops<T>::chiral_from64(int n, const uint4* src64, uint4* dst, cudaStr
 template <typename T>
 cudaError_t Ops<T>::pupdate(int n, int nrhs, long long vs, uint4* p, const uint4* v, const uint4* r,
                             const SolverState* st, int rev, cudaStream_t s) {
-    const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, VEC_BLOCK);
+    const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, vec_block<T>());
     { const cudaError_t le_ = launch_k(k_pupdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, p, v, r, st, rev); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
@@ -328,7 +333,7 @@ cudaError_t Ops<T>::pupdate(int n, int nrhs, long long vs, uint4* p, const uint4
 template <typename T>
 cudaError_t Ops<T>::supdate(int n, int nrhs, long long vs, uint4* r, const uint4* v, const SolverState* st,
                             int rev, cudaStream_t s) {
-    const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, VEC_BLOCK);
+    const int steps = (n + Stream<T>::SITES - 1) / Stream<T>::SITES, block = spread_block(steps, nrhs, vec_block<T>());
     { const cudaError_t le_ = launch_k(k_supdate<T>, stream_blocks(steps, block) * nrhs, block, 0, s, n, nrhs, vs, r, v, st, rev); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
@@ -339,7 +344,7 @@ cudaError_t Ops<T>::xr(int mode, int n, int nrhs, long long vs, uint4* x, uint4*
                        SolverState* st, RedCtx rc, int rev, cudaStream_t s) {
 #define WD_XR_CASE(M)                                                                                        \
     if (mode == M) {                                                                                         \
-        const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_xr<T, M>, n, block, nrhs);                            \
+        const int block = spread_block(n, nrhs, vec_block<T>()), nb = reduce_blocks((const void*)k_xr<T, M>, n, block, nrhs);                            \
         { const cudaError_t le_ = launch_k(k_xr<T, M>, nb * nrhs, block, 0, s, n, nrhs, vs, x, r, p, t, rstar, xr_src, xp_src, st, rc, rev); if (le_ != cudaSuccess) return le_; }   \
         return cudaGetLastError();                                                                           \
     }
@@ -353,7 +358,7 @@ cudaError_t Ops<T>::xr(int mode, int n, int nrhs, long long vs, uint4* x, uint4*
 template <typename T>
 cudaError_t Ops<T>::scale(int n, int nrhs, long long vs, uint4* r, uint4* x, const uint4* rstar, SolverState* st,
                           RedCtx rc, cudaStream_t s) {
-    const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_scale<T>, n, block, nrhs);
+    const int block = spread_block(n, nrhs, vec_block<T>()), nb = reduce_blocks((const void*)k_scale<T>, n, block, nrhs);
     { const cudaError_t le_ = launch_k(k_scale<T>, nb * nrhs, block, 0, s, n, nrhs, vs, r, x, rstar, st, rc); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
 }
@@ -361,7 +366,7 @@ cudaError_t Ops<T>::scale(int n, int nrhs, long long vs, uint4* r, uint4* x, con
 template <typename T>
 cudaError_t Ops<T>::rescale_in(int n, int nrhs, long long vs, long long vs64, const uint4* r64, uint4* r,
                                uint4* rstar, int ftz, SolverState* st, RedCtx rc, cudaStream_t s) {
-    const int block = spread_block(n, nrhs, VEC_BLOCK), nb = reduce_blocks((const void*)k_rescale_in<T>, n, block, nrhs);
+    const int block = spread_block(n, nrhs, vec_block<T>()), nb = reduce_blocks((const void*)k_rescale_in<T>, n, block, nrhs);
     k_rescale_in<T><<<nb * nrhs, block, 0, s>>>(n, nrhs, vs, vs64, r64, r, rstar, ftz, st, rc);
     return cudaGetLastError();
 }
