@@ -265,23 +265,73 @@ __device__ __forceinline__ void chiral_block_mul(const uint4* __restrict__ mat, 
         }
 }
 
+// Both blocks at once on FP32x2 pairs (S_+, S_-): they have the same layout, so
+// every product of the two is one packed operation (132 multiply-adds instead
+// of 264), term for term those of chiral_block_mul. For 16-bit storage, where
+// the pairs come out of the conversions: even-odd clover operator in FP16
+// arithmetic at 32^4 76.9 -> 75.5 us (FP32 storage: 137.5 -> 139.7, not taken).
+template <typename T>
+__device__ __forceinline__ void chiral_blocks_x2(const uint4* __restrict__ mat, int stride, int h,
+                                                 const float2 (&x)[12], float2 (&o)[12]) {
+    constexpr int N = Unit<T>::N;
+    constexpr int UB = 40 / N;   // units per block
+    int i = 0, j = 1;            // the off-diagonal element at hand
+#pragma unroll
+    for (int u = 0; u < UB; ++u) {
+        const uint4 p = __ldg(mat + (size_t)u * stride + h), m = __ldg(mat + (size_t)(UB + u) * stride + h);
+#pragma unroll
+        for (int e = u * N; e < (u + 1) * N; e += 2) {
+            const float2 a = make_float2(Unit<T>::get(p, e - u * N), Unit<T>::get(m, e - u * N));
+            const float2 b = make_float2(Unit<T>::get(p, e + 1 - u * N), Unit<T>::get(m, e + 1 - u * N));
+            if (e < 6) {         // two diagonal elements
+                o[2 * e] = __fmul2_rn(a, x[2 * e]);
+                o[2 * e + 1] = __fmul2_rn(a, x[2 * e + 1]);
+                o[2 * e + 2] = __fmul2_rn(b, x[2 * e + 2]);
+                o[2 * e + 3] = __fmul2_rn(b, x[2 * e + 3]);
+            } else if (e < 36) { // a + i b at (i, j): o_i += (a + i b) x_j ; o_j += (a - i b) x_i
+                const float2 nb = make_float2(-b.x, -b.y);
+                o[2 * i] = __ffma2_rn(a, x[2 * j], __ffma2_rn(nb, x[2 * j + 1], o[2 * i]));
+                o[2 * i + 1] = __ffma2_rn(a, x[2 * j + 1], __ffma2_rn(b, x[2 * j], o[2 * i + 1]));
+                o[2 * j] = __ffma2_rn(a, x[2 * i], __ffma2_rn(b, x[2 * i + 1], o[2 * j]));
+                o[2 * j + 1] = __ffma2_rn(a, x[2 * i + 1], __ffma2_rn(nb, x[2 * i], o[2 * j + 1]));
+                if (++j == 6) {
+                    ++i;
+                    j = i + 1;
+                }
+            }
+        }
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ void mat_mul_chiral(const uint4* __restrict__ mat, int stride, int h,
                                                const typename Unit<T>::C (&v)[24], typename Unit<T>::C (&out)[24]) {
     typedef typename Unit<T>::C C;
-    constexpr int UB = 40 / Unit<T>::N;
-    C xp[12], xm[12], op[12], om[12];
+    if constexpr (sizeof(T) == 2) {
+        float2 x[12], o[12];
 #pragma unroll
-    for (int i = 0; i < 12; ++i) {   // spin pair (k, k + 2), colour: reals 6 k + 2 a + re/im
-        xp[i] = v[i] - v[12 + i];
-        xm[i] = v[i] + v[12 + i];
-    }
-    chiral_block_mul<T>(mat, stride, h, 0, xp, op);
-    chiral_block_mul<T>(mat, stride, h, UB, xm, om);
+        for (int i = 0; i < 12; ++i) x[i] = make_float2(v[i] - v[12 + i], v[i] + v[12 + i]);
+        chiral_blocks_x2<T>(mat, stride, h, x, o);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) {
-        out[i] = op[i] + om[i];
-        out[12 + i] = om[i] - op[i];
+        for (int i = 0; i < 12; ++i) {
+            out[i] = o[i].x + o[i].y;
+            out[12 + i] = o[i].y - o[i].x;
+        }
+    } else {
+        constexpr int UB = 40 / Unit<T>::N;
+        C xp[12], xm[12], op[12], om[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {   // spin pair (k, k + 2), colour: reals 6 k + 2 a + re/im
+            xp[i] = v[i] - v[12 + i];
+            xm[i] = v[i] + v[12 + i];
+        }
+        chiral_block_mul<T>(mat, stride, h, 0, xp, op);
+        chiral_block_mul<T>(mat, stride, h, UB, xm, om);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+            out[i] = op[i] + om[i];
+            out[12 + i] = om[i] - op[i];
+        }
     }
 }
 

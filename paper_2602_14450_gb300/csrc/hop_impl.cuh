@@ -345,11 +345,14 @@ __device__ __forceinline__ void link_mul_pair(const uint4 (&u)[LinkFmt<T, R>::GR
 // Launch bounds of hop_kernel: the FP16 look-ahead kernels without a fused
 // reduction fit 72 registers (7 blocks of 128 threads per SM; measured 3%
 // faster, while BF16 there is 6% slower), the other 16-bit kernels keep 80
-// (3 blocks of 256); FP32 128 and FP64 255 registers.
+// (3 blocks of 256), with a clover block 102 (5 of 128: even-odd operator at
+// 24^3 x 48 FP16 58.3 -> 57.3, BF16 62.8 -> 60.5 us); FP32 128 and FP64 255
+// registers.
 template <typename T, int RED, bool PF, bool MAT = false> struct HopBounds {
     static constexpr bool LEAN = std::is_same<T, __half>::value && PF && RED == RED_NONE && !MAT;
-    static constexpr int THREADS = LEAN ? 128 : 256;
-    static constexpr int MIN_BLOCKS = LEAN ? 7 : sizeof(T) == 2 ? (PF ? 3 : 2) : sizeof(T) == 4 ? 2 : 1;
+    static constexpr bool BLOCKS = sizeof(T) == 2 && PF && MAT;
+    static constexpr int THREADS = LEAN || BLOCKS ? 128 : 256;
+    static constexpr int MIN_BLOCKS = LEAN ? 7 : BLOCKS ? 5 : sizeof(T) == 2 ? (PF ? 3 : 2) : sizeof(T) == 4 ? 2 : 1;
 };
 
 template <typename T, int R, int EPI, int RED, bool PF, bool PAIR = false, bool MAT = false>

@@ -94,6 +94,26 @@ __device__ __forceinline__ void spin_mul_add_p(const float2* w, const float* phi
             }
         }
 }
+// The same on FP32x2 pairs (re, im), term for term: w holds (c.x, c.x, -c.y, c.y), phi and acc complex numbers.
+__device__ __forceinline__ void spin_mul_add_x2(const float4* w, const float2* phi, float2 (&acc)[12]) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        float2 f[3], g[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            f[a] = phi[3 * t + a];
+            g[a] = make_float2(f[a].y, f[a].x);
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const float4 c = w[4 * s + t];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                acc[3 * s + a] = __ffma2_rn(make_float2(c.z, c.w), g[a],
+                                            __ffma2_rn(make_float2(c.x, c.y), f[a], acc[3 * s + a]));
+        }
+    }
+}
 __device__ __forceinline__ void spin_mul_add(const float2* w, const float (&phi)[24], float (&acc)[24]) {
     spin_mul_add_p(w, phi, acc);
 }
@@ -126,8 +146,7 @@ __global__ void k_ptc_collapse(const float* w, float2* V) {
 }
 
 constexpr int S1_SITES = 32;                // sites per block of the first pass
-constexpr int S1_STRIDE = 8 * 24 + 1;       // floats per site of its transport tile (padded)
-constexpr int S1_VROW = 8 * 16 + 1;         // float2 per k2 row of its V tile (padded)
+constexpr int S1_STRIDE = 8 * 24 + 2;       // floats per site of its transport tile (padded, pairs aligned)
 
 // First pass on the odd sites y: the eight transports T_{1+d} psi(y) (warp mu
 // computes directions 2 mu and 2 mu + 1 for the block's 32 sites) go to shared
@@ -139,11 +158,11 @@ __global__ void __launch_bounds__(128) k_ptc_s1(Geom g, const uint4* in_e, uint4
     if (guarded(guard, GUARD_INNER)) return;
     in_e += blockIdx.y * (long long)Spinor<TIN>::UNITS * g.Vh;      // sample blockIdx.y, vectors back to back
     phi += blockIdx.y * 8 * pvs;
-    __shared__ float ts[S1_SITES * S1_STRIDE];
-    __shared__ float2 vs[8 * S1_VROW];
+    __shared__ __align__(16) float ts[S1_SITES * S1_STRIDE];
+    __shared__ float4 vs[64 * 16];   // V[1 + a][1 + b] at 16 (8 a + b), as spin_mul_add_x2 takes it
     for (int i = threadIdx.x; i < 64 * 16; i += blockDim.x) {
-        const int a = i / 128, b = i % 128;     // a = k2 - 1, b = 16 (k1 - 1) + e
-        vs[a * S1_VROW + b] = V[((1 + a) * 9 + 1 + b / 16) * 16 + b % 16];
+        const float2 c = V[((1 + i / 128) * 9 + 1 + (i / 16) % 8) * 16 + i % 16];
+        vs[i] = make_float4(c.x, c.x, -c.y, c.y);
     }
     __syncthreads();
     const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -175,11 +194,18 @@ __global__ void __launch_bounds__(128) k_ptc_s1(Geom g, const uint4* in_e, uint4
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int d2 = 2 * mu + j;
+                float2 sum[12];
+#pragma unroll
+                for (int i = 0; i < 12; ++i) sum[i] = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int k1 = 0; k1 < 8; ++k1)
+                    spin_mul_add_x2(&vs[16 * (8 * d2 + k1)], reinterpret_cast<const float2*>(mine + 24 * k1), sum);
                 float acc[24];
 #pragma unroll
-                for (int i = 0; i < 24; ++i) acc[i] = 0.f;
-#pragma unroll 1
-                for (int k1 = 0; k1 < 8; ++k1) spin_mul_add_p(&vs[d2 * S1_VROW + 16 * k1], mine + 24 * k1, acc);
+                for (int i = 0; i < 12; ++i) {
+                    acc[2 * i] = sum[i].x;
+                    acc[2 * i + 1] = sum[i].y;
+                }
                 store_spinor<TPHI>(phi + (size_t)d2 * pvs, g.Vh, h, acc);
             }
         }
@@ -439,7 +465,7 @@ __global__ void __launch_bounds__(256) k_ptc_corr_sum(int blocks, int n, const f
     __shared__ float2 sh[8][32];
     const int i = blockIdx.x * 32 + (threadIdx.x & 31), q = threadIdx.x >> 5;
     F2 t = {0.f, 0.f};
-#pragma unroll 4
+#pragma unroll 16
     for (int b = q; b < blocks; b += 8) t = f2_add(t, F2{part[(size_t)b * n + i], 0.f});
     sh[q][threadIdx.x & 31] = make_float2(t.hi, t.lo);
     __syncthreads();
