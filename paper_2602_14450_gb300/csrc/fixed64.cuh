@@ -7,17 +7,17 @@
 // fixed point, three integer multiply-adds for one FP64 one:
 //
 //   link     u = 2^-61 (u1 2^32 + u0)                     signed 32-bit digits u1, u0
-//   spinor   p = 2^(E-1081) * (a 60-bit integer)           E: the largest biased exponent of the site's neighbour
-//                                                          reals so far (acc is shifted when it grows)
+//   spinor   p = 2^(E-1081) * (a 60-bit integer)           E: one above the largest biased exponent of a
+//                                                          neighbour, raised (and acc shifted) when one exceeds E
 //   half spinor h = p +- p' = 2^(E-1081) (h1 2^32 + h0)
 //   u h      = 2^(E-1078) (u1 h1 + (u1 h0 + u0 h1) 2^-32)  (u0 h0 is below the last unit)
 //   H        = 2^(E-1078) * (64-bit sum over the eight directions)
 //
-// Errors, in units of 2^(E-1078), at most 2^-55 of the largest neighbour real:
+// Errors, in units of 2^(E-1078), at most 2^-54 of the largest neighbour real:
 // a product of a link row with a column is off by at most 3.5 (spinor reals cut
 // at 1/8 each: 0.6; u0 h0 left out: 1.5; link entries: 0.2; its own rounding
 // and a shift: 1), typically 0.3, and a site's sum is rounded once more to
-// FP64. The relative error of a hop of Gaussian fields is 0.92e-16 against
+// FP64. The relative error of a hop of Gaussian fields is 0.93e-16 against
 // 1.0e-16 in FP64 arithmetic (~25 roundings at 2^-53).
 //
 // Bounds (rows of unit norm, |h| < 2^60): |sum u1 h0| <= sqrt(6) 2^29 2^31 and

@@ -223,8 +223,8 @@ __device__ __forceinline__ void epilogue16x2(const HopParams& P, uint4* vout, co
         }
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
-            part[0] += rs[i].x * o[i].x + rs[i].y * o[i].y;
-            part[1] += rs[i].x * o[i].y - rs[i].y * o[i].x;
+            add_fused(part[0], rs[i].x, o[i].x, rs[i].y, o[i].y);
+            sub_fused(part[1], rs[i].x, o[i].y, rs[i].y, o[i].x);
         }
     } else if constexpr (RED == RED_TS) {   // (o, q), (o, o), (q, q); q = r* if given, else y
         float2 q2[12];
@@ -241,10 +241,10 @@ __device__ __forceinline__ void epilogue16x2(const HopParams& P, uint4* vout, co
         }
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
-            part[0] += o[i].x * q2[i].x + o[i].y * q2[i].y;
-            part[1] += o[i].x * q2[i].y - o[i].y * q2[i].x;
-            part[2] += o[i].x * o[i].x + o[i].y * o[i].y;
-            part[3] += q2[i].x * q2[i].x + q2[i].y * q2[i].y;
+            add_fused(part[0], o[i].x, q2[i].x, o[i].y, q2[i].y);
+            sub_fused(part[1], o[i].x, q2[i].y, o[i].y, q2[i].x);
+            add_fused(part[2], o[i].x, o[i].x, o[i].y, o[i].y);
+            add_fused(part[3], q2[i].x, q2[i].x, q2[i].y, q2[i].y);
         }
     } else if constexpr (RED == RED_NORM) {
 #pragma unroll

@@ -181,12 +181,14 @@ __global__ void __launch_bounds__(HOP64_THREADS, HOP64_BLOCKS) hop64_kernel(cons
                 continue;
             }
             if (En > E) {
+                // one binade above, which most later neighbours stay below: fewer shifts (913 -> 896 us for D_W)
+                const int Ek = min(En + 1, fx::E_MAX);
                 if (E) {
-                    const int sh = min(En - E, 63);
+                    const int sh = min(Ek - E, 63);
 #pragma unroll
                     for (int i = 0; i < 24; ++i) acc[i] >>= sh;
                 }
-                E = En;
+                E = Ek;
             }
             if ((neg >> d) & 1u) {
 #pragma unroll

@@ -12,17 +12,19 @@
 
 namespace wd {
 
-// s += a b + c d. FP64 takes two fused multiply-adds: its pipe (2 per cycle and SM) bounds the FP64 vector kernels
-// and reductions, and the expression as written is three operations there.
+// s += a b + c d and s += a b - c d. FP64 takes two fused multiply-adds: its pipe (2 per cycle and SM) bounds the
+// FP64 vector kernels and reductions, and the expression as written is three operations there.
 template <typename C> __device__ __forceinline__ void add_products(C& s, C a, C b, C c, C d) { s += a * b + c * d; }
 template <> __device__ __forceinline__ void add_products<double>(double& s, double a, double b, double c, double d) {
     s = fma(c, d, fma(a, b, s));
 }
-// s += a b - c d, likewise.
 template <typename C> __device__ __forceinline__ void sub_products(C& s, C a, C b, C c, C d) { s += a * b - c * d; }
 template <> __device__ __forceinline__ void sub_products<double>(double& s, double a, double b, double c, double d) {
     s = fma(-c, d, fma(a, b, s));
 }
+// The same as two fused multiply-adds in FP32 (the dot products of the FP16-arithmetic hop).
+__device__ __forceinline__ void add_fused(float& s, float a, float b, float c, float d) { s = fma(c, d, fma(a, b, s)); }
+__device__ __forceinline__ void sub_fused(float& s, float a, float b, float c, float d) { s = fma(-c, d, fma(a, b, s)); }
 
 enum Epi { EPI_H = 0, EPI_Y = 1, EPI_YZ = 2 };
 enum Red { RED_NONE = 0, RED_RSV = 1, RED_TS = 2, RED_NORM = 3 };
