@@ -55,7 +55,7 @@ def test_fixed_point_hop_matches_fp64_arithmetic(dims, bc, kind):
         assert torch.equal(torch.isnan(x), torch.isnan(y))
         assert torch.equal(torch.isinf(x), torch.isinf(y)) and torch.equal(x[torch.isinf(x)], y[torch.isinf(y)])
         x, y = (torch.where(torch.isfinite(z), z, 0.0) for z in (x, y))
-        # 36 fixed-point units of at most 2^-55 of the site's largest neighbour, ~25 roundings of the FP64 sum;
+        # 36 fixed-point units of at most 2^-54 of the site's largest neighbour, ~25 roundings of the FP64 sum;
         # the site's largest neighbour bounds every result of the site, and is at most the lattice's
         size = lex.cpu().reshape(-1, 24)
         size = size[torch.isfinite(size)].abs().max()
