@@ -23,6 +23,7 @@ static __device__ __noinline__ void hop64_site(const HopParams& P, const uint4* 
     for (int d = 0; d < 8; ++d) {
         const int mu = d >> 1;
         const bool fwd = (d & 1) == 0;
+        if (((wm >> d) & 1u) && ((g.part >> mu) & 1u)) continue;   // leaves the sub-lattice
         double nb[24], hs[12], chi[12];
         uint4 u[9];
         load_spinor<double>(vin, g.Vh, nbr[d], nb);
@@ -123,10 +124,11 @@ __global__ void __launch_bounds__(HOP64_THREADS, HOP64_BLOCKS) hop64_kernel(cons
         unsigned neg;          // directions whose hop carries a boundary phase -1
         {
             int nbr[8];
-            neg = site_neighbours(g, P.parity, h, nbr);
+            neg = site_neighbours(g, P.parity, h, nbr);   // those that wrap around
 #pragma unroll
             for (int d = 0; d < 8; ++d) {
-                nbs[d][threadIdx.x] = nbr[d];
+                // -1: a hop that leaves the sub-lattice of a split direction has no neighbour here
+                nbs[d][threadIdx.x] = ((neg >> d) & 1u) && ((g.part >> (d >> 1)) & 1u) ? -1 : nbr[d];
                 if (g.bc[d >> 1] > 0) neg &= ~(1u << d);
             }
         }
@@ -144,9 +146,15 @@ __global__ void __launch_bounds__(HOP64_THREADS, HOP64_BLOCKS) hop64_kernel(cons
         bool bad = false;
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
-            const int mu = d >> 1;
+            const int mu = d >> 1, hn = nbs[d][threadIdx.x];
+            if (hn < 0) {
+                if (d + 1 < 8) copy_links(d + 1);
+                else cp_async_commit();
+                cp_async_wait<1>();          // the next copy reuses the slot of the one before this
+                continue;
+            }
             // upper spins p (of the t hops: the pair the projector keeps) and their partners q
-            const uint4* np = vin + nbs[d][threadIdx.x];
+            const uint4* np = vin + hn;
             const uint4* pp = np + (size_t)(d == 6 ? 6 : 0) * Vh;
             uint4 p[6], q[6];
 #pragma unroll
