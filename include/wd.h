@@ -64,8 +64,10 @@ enum wd_status {
 };
 
 /* Storage precisions of packed vectors and links. Arithmetic is FP32 for
- * FP32/FP16/BF16 storage and FP64 for FP64 storage, where the hop of SU(3)
- * links is summed in 64-bit fixed point (no less accurate). */
+ * FP32/FP16/BF16 storage and FP64 for FP64 storage. The FP64 hop of SU(3)
+ * links is summed in 64-bit fixed point at the sites where the error bound of
+ * every real is then no larger than that of FP64 arithmetic (15 x 2^-53 times
+ * the sum of the sizes of its products), in FP64 arithmetic at all others. */
 enum wd_prec { WD_FP64 = 0, WD_FP32 = 1, WD_FP16 = 2, WD_BF16 = 3 };
 
 /* Link formats: 18 reals (full 3x3) or 12 reals (two rows; the third row is

@@ -7,18 +7,30 @@
 // fixed point, three integer multiply-adds for one FP64 one:
 //
 //   link     u = 2^-61 (u1 2^32 + u0)                     signed 32-bit digits u1, u0
-//   spinor   p = 2^(E-1081) * (a 60-bit integer)           E: one above the largest biased exponent of a
-//                                                          neighbour, raised (and acc shifted) when one exceeds E
+//   spinor   p = 2^(E-1081) * (a 60-bit integer)           E: largest biased exponent of a neighbour so far (acc is
+//                                                          shifted when a later one exceeds it)
 //   half spinor h = p +- p' = 2^(E-1081) (h1 2^32 + h0)
 //   u h      = 2^(E-1078) (u1 h1 + (u1 h0 + u0 h1) 2^-32)  (u0 h0 is below the last unit)
 //   H        = 2^(E-1078) * (64-bit sum over the eight directions)
 //
-// Errors, in units of 2^(E-1078), at most 2^-54 of the largest neighbour real:
-// a product of a link row with a column is off by at most 3.5 (spinor reals cut
-// at 1/8 each: 0.6; u0 h0 left out: 1.5; link entries: 0.2; its own rounding
-// and a shift: 1), typically 0.3, and a site's sum is rounded once more to
-// FP64. The relative error of a hop of Gaussian fields is 0.93e-16 against
-// 1.0e-16 in FP64 arithmetic (~25 roundings at 2^-53).
+// Errors, in units of 2^(E-1078), at most 2^-55 of the largest neighbour real:
+// a product of a link row with a column is off by at most 2.8 (spinor reals cut
+// at 1/8 each: 0.6; u0 h0 left out: 1.5; link entries: 0.2; its own rounding:
+// 0.5), of a t hop, doubled, by 4.8; six of the first and one of the second
+// make 21.6 per real of the sum, shifts of the sum less than 2 more. Then the
+// sum is rounded once to FP64.
+//
+// These errors go with the largest neighbour of the site, those of FP64
+// arithmetic with each real by itself: 14 x 2^-53 times the sum S of the sizes
+// of its products (a rounding of the projection, six of the colour row, seven
+// of the sum). So a real may be formed here when S >= 1.69 x 2^53 units, where
+// 14 x 2^-53 S is 23.6 units. hop64_kernel sums the products of the entries' sizes
+// rounded down, links to 2^-5 and half spinors to 2^(E-1027), which S is never
+// below; SIZE_MIN is that in its units of 2^(E-1032). On rough links 1 site in
+// 10^6 fails; components fed by small spinor parts or small link entries alone do,
+// and reals that are zero.
+// The relative error of a hop of Gaussian fields is 0.92e-16 against 1.0e-16
+// in FP64 arithmetic.
 //
 // Bounds (rows of unit norm, |h| < 2^60): |sum u1 h0| <= sqrt(6) 2^29 2^31 and
 // |sum u0 h1| <= 6 2^31 2^28, together 6.3e18 < 2^63; a product is at most
@@ -40,6 +52,9 @@ namespace fx {
 // Neighbours whose largest biased exponent lies outside [E_MIN, E_MAX] (and are not zero) take the FP64 path of
 // the site: below, the result could be subnormal; above, it could overflow or the input is not finite.
 constexpr int E_MIN = 70, E_MAX = 2030;
+// The least size of a real's products, in units of 2^(E-1032), at which fixed point is as exact as FP64 arithmetic
+// (above). Their sum stays below 2^16: 6 x 32 x 64 sqrt(6) + 2 x 32 x 32 sqrt(6).
+constexpr unsigned SIZE_MIN = 216;
 
 // v >> s, zero for s >= 64.
 __host__ __device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned s) {

@@ -112,6 +112,7 @@ inline void apply_tuning(const wd_handle* h, int prec, int recon, HopParams& P) 
     }
     P.arith16 = (prec == WD_FP16 && h->arith16) ? 1 : 0;
     P.fixed64 = (prec == WD_FP64 && recon == 18 && h->fixed64) ? 1 : 0;
+    P.U64 = h->U64;
     P.wait_rounds = h->wait_rounds;
     for (int f = 0; f < 2; ++f) {
         P.rhs_group[f] = P.arith16 ? h->tune_rhs[recon == 12 ? 0 : 1][f] : 0;

@@ -247,11 +247,7 @@ __device__ __forceinline__ void hop_epilogue(const HopParams& P, uint4* vout, co
         C zv[24];
         load_spinor<T>(vz, Vh, h, zv);
 #pragma unroll
-        for (int i = 0; i < 24; ++i) {
-            // FP64 residual r = (y - x) + a H: the two large terms are subtracted before the small one is added
-            if (sizeof(C) == 8 && unit_b && P.c == -1.0) o[i] = fma(ca, acc[i], yv[i] - zv[i]);
-            else o[i] += cc * zv[i];
-        }
+        for (int i = 0; i < 24; ++i) o[i] += cc * zv[i];
     }
     store_spinor<T>(vout, Vh, h, o, ftz);
 

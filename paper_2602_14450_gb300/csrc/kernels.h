@@ -60,6 +60,7 @@ struct HopParams {
     int rhs_smem[2];           // ... and 1 = the site's links in shared memory instead of registers
     int rev;                   // 1 = take the sites from the last to the first (sweep_site; FP16 arithmetic)
     int fixed64;               // FP64, 18-real: the links are fixed-point digits (hop64_kernel)
+    const double* U64;         // ... and the FP64 links in the host layout, for sites that take FP64 arithmetic
     int spt;                   // FP16 arithmetic, plain hop: sites per thread (grid-stride; 0 or 1 = one site)
 };
 

@@ -59,6 +59,7 @@ extern "C" int wd_tune(wd_handle* h, int prec, int recon, int nrhs, void* stream
     P.a = 1.0;
     P.b = 1.0;
     P.fixed64 = (prec == WD_FP64 && recon == 18 && h->fixed64) ? 1 : 0;
+    P.U64 = h->U64;
     P.guard_kind = GUARD_NONE;
     P.rc = red_ctx(h, ST_NONE);   // the last block of a reduction finds no scalar stage to run
     cudaEvent_t e0, e1;

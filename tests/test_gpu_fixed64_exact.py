@@ -11,7 +11,7 @@ import pytest
 import torch
 
 from oracle.gamma import projectors
-from paper_2602_14450_gb300 import synth
+from paper_2602_14450_gb300 import synth, wd
 from tests.gpu_util import lattice, packed
 
 pytestmark = pytest.mark.gpu
@@ -71,6 +71,67 @@ def check(got, want):
     for site, reals in want.items():
         for i, (v, m) in enumerate(reals):
             assert abs(F(got[site][i]) - v) <= UNIT * m, (site, i, got[site][i], float(v), float(m))
+
+
+def smooth(dims, eps, seed):
+    """SU(3) links with off-diagonal entries of size eps around diagonal phases."""
+    u = synth.gauge_random(dims, eps, seed=seed)
+    ph = synth.gaussian_source(dims, seed=seed + 1)[..., 0, :2].real
+    a, b = ph[..., 0], ph[..., 1]
+    d = torch.polar(torch.ones_like(torch.stack([a, b, -a - b], -1)), torch.stack([a, b, -a - b], -1))
+    return d[None, ..., :, None] * u
+
+
+def fields(dims, kind):
+    """Links and spinors of a kind."""
+    u = synth.gauge_random(dims, 0.5, seed=9)
+    psi = synth.gaussian_source(dims, seed=4)
+    v = psi.reshape(-1, 4, 3)
+    if kind == "small entries":     # one colour only: the others are fed by small link entries alone
+        u = smooth(dims, 1e-9, 9)
+        v[:, :, 1:] = 0.0
+    elif kind == "tiny entries":    # below the last bit of a fixed-point link
+        u = smooth(dims, 1e-20, 9)
+        v[:, :, 1:] = 0.0
+    elif kind == "unit links":
+        u = torch.eye(3, dtype=u.dtype).expand_as(u).contiguous()
+        v[:, :, 2] *= 1e-8
+    elif kind == "spins":           # two spins much smaller
+        v[:, 2:] *= 1e-8
+    elif kind == "one spin":
+        v[:, 1:] = 0.0
+    elif kind == "time slices":     # large t neighbours, which feed two spins of a site
+        psi[::2] *= 1e-8
+    elif kind == "spread":          # sites of very different size
+        v *= 10.0 ** (30 * torch.rand(v.shape[0], 1, 1, generator=torch.Generator().manual_seed(2)).double() - 15)
+    elif kind == "point":
+        v[1:] = 0.0
+        v[0, 1:] = 0.0
+    elif kind == "small":           # reals at the lower end of the fixed-point range
+        v *= 2.0 ** -950
+    elif kind == "large":
+        v *= 2.0 ** 1000
+    return u, psi
+
+
+KINDS = ["gauss", "small entries", "tiny entries", "unit links", "spins", "one spin", "time slices", "spread", "point",
+         "small", "large"]
+
+
+@pytest.mark.parametrize("dims,bc", [((2, 2, 2, 4), (1, 1, 1, -1)), ((4, 2, 6, 2), (-1, 1, -1, 1))])
+@pytest.mark.parametrize("kind", KINDS)
+def test_every_component_within_the_bound_of_fp64_arithmetic(dims, bc, kind):
+    u, psi = fields(dims, kind)
+    lat = lattice(u, 0.1, dims, bc)
+    dev = lat.unitarity()
+    assert max(dev) < 1e-6
+    for op, p in ((wd.WD_OP_HOP_EO, 0), (wd.WD_OP_HOP_OE, 1)):
+        src, dst = packed(lat, "fp64"), packed(lat, "fp64")
+        lat.pack("fp64", 1 - p, lex(psi), src)
+        lat.apply("fp64", 18, op, src, dst)
+        got = torch.zeros_like(lex(psi))
+        lat.unpack("fp64", p, dst, got)
+        check(got.cpu().reshape(-1, 24).tolist(), exact_hop(u, psi, p, bc))
 
 
 def lex(psi):
