@@ -309,6 +309,9 @@ __global__ void __launch_bounds__(192) k_clover_build(Geom g, Field f, double ck
 // copies are dropped and rebuilt on first use.
 int clover_build(wd_handle* h) {
     const size_t bytes = (size_t)h->g.Vh * 40 * 16;
+    // blocks that are there are rewritten in place, the lower precisions on their next use: work on any stream that
+    // still reads them has to be done
+    if (h->clov64[0][0]) WD_CUDA(h, cudaDeviceSynchronize());
     uint4* b[4];
     const char* names[4] = {"clov.fwd64.e", "clov.fwd64.o", "clov.inv64.e", "clov.inv64.o"};
     for (int i = 0; i < 4; ++i) {
