@@ -17,6 +17,7 @@
 // Training: for L = sum |M v - y|^2/|y|^2 + mu |A M v - v|^2/|v|^2 the weight
 // gradients dL/dRe W + i dL/dIm W follow from the 8 x 8 (+ 1) correlations of
 // the transported loss gradient with the transported input (below).
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -732,8 +733,10 @@ static cudaError_t apply_A_f32(wd_handle* h, int n, const uint4* in, uint4* out,
     return Ops<float>::hop(18, EPI_Y, RED_NONE, P, s);
 }
 
-// Bytes of workspace of a chunk of samples (13 vectors each); a larger batch goes through chunk by chunk.
+// Bytes of workspace of a chunk of samples (13 vectors each); a larger batch goes through chunk by chunk. The samples
+// of a chunk are gridDim.y of its launches, at most 65535.
 constexpr size_t PTC_CHUNK_BYTES = (size_t)2 << 30;
+constexpr size_t PTC_CHUNK_SAMPLES = 65535;
 
 int ptc_grad(wd_handle* h, int n, const float* v, const float* y, double mu, double* loss, cudaStream_t s) {
     PtcBufs B;
@@ -744,7 +747,7 @@ int ptc_grad(wd_handle* h, int n, const float* v, const float* y, double mu, dou
     const Geom& g = h->g;
     const size_t vb = vec_bytes(h, WD_FP32);
     const long long vs = (long long)spinor_units(WD_FP32) * g.Vh;   // 16-byte units of a vector
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)n, PTC_CHUNK_BYTES / (13 * vb)));
+    const int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)n, PTC_CHUNK_BYTES / (13 * vb), PTC_CHUNK_SAMPLES}));
     uint4* m = (uint4*)workspace(h, "ptc.vm", vb * chunk);
     uint4* am = (uint4*)workspace(h, "ptc.vam", vb * chunk);
     uint4* t1 = (uint4*)workspace(h, "ptc.vt1", vb * chunk);
