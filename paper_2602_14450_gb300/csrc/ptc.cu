@@ -511,13 +511,24 @@ __device__ __forceinline__ void add_square(F2& s, float x) {
     const float p = __fmul_rn(x, x);
     s = f2_add(s, F2{p, __fmaf_rn(x, x, -p)});
 }
+// Whether the squares of q, their rounding errors and their sum over any lattice stay in FP32's range.
+__device__ __forceinline__ bool ordinary(float x) {
+    const float a = fabsf(x);
+    return (a >= 0x1p-50f && a <= 0x1p50f) || x == 0.f;
+}
+__device__ __forceinline__ bool ordinary(const float4& q) {
+    return ordinary(q.x) && ordinary(q.y) && ordinary(q.z) && ordinary(q.w);
+}
 
 // For sample blockIdx.y: t = gamma5 e2 with e2 = a - v (a = A m), and this
-// block's share of |v|^2, |y|^2, |m - y|^2, |e2|^2 (FP32 pairs, about 48 bits).
+// block's share of |v|^2, |y|^2, |m - y|^2, |e2|^2 (FP32 pairs, about 48 bits; in FP64 the values outside the
+// range of FP32 squares).
 __global__ void __launch_bounds__(256) k_ptc_resid(int Vh, long long vs, const float4* v, const float4* y,
                                                    const float4* m, const float4* a, float4* t, double* part) {
     const long long o = blockIdx.y * vs;
     F2 s[4] = {};
+    double far[4] = {0.0, 0.0, 0.0, 0.0};
+    bool any = false;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < vs; i += (long long)gridDim.x * blockDim.x) {
         const float4 vv = v[o + i], yv = y[o + i], mv = m[o + i], av = a[o + i];
         const float4 e1 = make_float4(mv.x - yv.x, mv.y - yv.y, mv.z - yv.z, mv.w - yv.w);
@@ -525,18 +536,30 @@ __global__ void __launch_bounds__(256) k_ptc_resid(int Vh, long long vs, const f
         // (g5 f)_s = -f_{s xor 2}: spins 0, 1 are units 0..2 of a site, spins 2, 3 units 3..5
         t[o + (i < vs / 2 ? i + vs / 2 : i - vs / 2)] = make_float4(-e2.x, -e2.y, -e2.z, -e2.w);
         const float4 q[4] = {vv, yv, e1, e2};
+        if (ordinary(vv) && ordinary(yv) && ordinary(e1) && ordinary(e2)) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            add_square(s[k], q[k].x);
-            add_square(s[k], q[k].y);
-            add_square(s[k], q[k].z);
-            add_square(s[k], q[k].w);
+            for (int k = 0; k < 4; ++k) {
+                add_square(s[k], q[k].x);
+                add_square(s[k], q[k].y);
+                add_square(s[k], q[k].z);
+                add_square(s[k], q[k].w);
+            }
+        } else {
+            any = true;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                far[k] = fma((double)q[k].x, (double)q[k].x, far[k]);
+                far[k] = fma((double)q[k].y, (double)q[k].y, far[k]);
+                far[k] = fma((double)q[k].z, (double)q[k].z, far[k]);
+                far[k] = fma((double)q[k].w, (double)q[k].w, far[k]);
+            }
         }
     }
     block_sum<4>(s);
+    if (__syncthreads_or(any)) block_sum<4>(far);
     if (threadIdx.x == 0)
         for (int k = 0; k < 4; ++k)
-            part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + k] = (double)s[k].hi + (double)s[k].lo;
+            part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + k] = ((double)s[k].hi + (double)s[k].lo) + far[k];
 }
 
 // dots[sample][4] = the sums of k_ptc_resid over its nb blocks, in a fixed order (one warp per sample).

@@ -30,3 +30,16 @@ def test_more_samples_than_a_launch_takes(dims):
     rows = 70000 * 24 * 3 / 608
     g = g.double()
     assert torch.linalg.vector_norm(gm.double() - 10000 * g) <= rows * 6e-8 * 10000 * torch.linalg.vector_norm(g)
+
+
+# 2^60, 2^-75: squares beyond FP32; 2^-45: their rounding errors; 2^49: above and below the border at once
+@pytest.mark.parametrize("k", [60, 49, -45, -75])
+def test_loss_does_not_depend_on_the_scale_of_the_samples(k):
+    dims = (4, 4, 6, 10)
+    lat = lattice(synth.gauge_random(dims, 0.5, seed=31), 0.12, dims)
+    lat.precond_set(bf16_weights(seed=32)[0])
+    v, y = samples(lat, dims, 3)
+    want, _ = lat.precond_grad(v, y, 0.7)
+    got, _ = lat.precond_grad(v * 2.0 ** k, y * 2.0 ** k, 0.7)
+    # M, A and the residuals scale exactly; the sums of squares are good to 2^-44
+    assert abs(got - want) <= 1e-12 * want
