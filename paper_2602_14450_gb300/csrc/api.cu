@@ -92,6 +92,15 @@ void* workspace(wd_handle* h, const std::string& name, size_t bytes) {
     return b.p;
 }
 
+void drop_workspace(wd_handle* h, const std::string& name) {
+    Buffer& b = h->ws[name];
+    if (!b.p) return;
+    cudaDeviceSynchronize();
+    cudaFree(b.p);
+    b = Buffer{};
+    ++h->gen;   // captured solver graphs may hold its address
+}
+
 int* lower_err(wd_handle* h) {
     if (!h->herr) {
         if (cudaHostAlloc((void**)&h->herr, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {

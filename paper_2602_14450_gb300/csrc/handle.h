@@ -89,6 +89,8 @@ int fail(wd_handle* h, int code, const char* fmt, ...);
 int cuda_fail(wd_handle* h, cudaError_t e, const char* what);
 // Device buffer `name` of at least `bytes` (reallocated, and gen bumped, when too small).
 void* workspace(wd_handle* h, const std::string& name, size_t bytes);
+// Frees a named workspace, once the device is done with it.
+void drop_workspace(wd_handle* h, const std::string& name);
 // Scalar state, partials and tickets for `nrhs` right-hand sides.
 int ensure_solver_state(wd_handle* h, int nrhs);
 int ensure_links(wd_handle* h, int prec, int recon, const uint4** even, const uint4** odd);

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "blas_impl.cuh"
+#include "chunk.h"
 #include "handle.h"
 
 namespace wd {
@@ -770,23 +771,35 @@ int ptc_grad(wd_handle* h, int n, const float* v, const float* y, double mu, dou
     const Geom& g = h->g;
     const size_t vb = vec_bytes(h, WD_FP32);
     const long long vs = (long long)spinor_units(WD_FP32) * g.Vh;   // 16-byte units of a vector
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>({(size_t)n, PTC_CHUNK_BYTES / (13 * vb), PTC_CHUNK_SAMPLES}));
-    uint4* m = (uint4*)workspace(h, "ptc.vm", vb * chunk);
-    uint4* am = (uint4*)workspace(h, "ptc.vam", vb * chunk);
-    uint4* t1 = (uint4*)workspace(h, "ptc.vt1", vb * chunk);
-    uint4* t2 = (uint4*)workspace(h, "ptc.vt2", vb * chunk);
-    uint4* gv = (uint4*)workspace(h, "ptc.vg", vb * chunk);
-    uint4* phi = (uint4*)workspace(h, "ptc.phi32", vb * 8 * chunk);
+    const int want = (int)std::max<size_t>(1, std::min<size_t>({(size_t)n, PTC_CHUNK_BYTES / (13 * vb), PTC_CHUNK_SAMPLES}));
     const int rb = (int)std::max<long long>(1, std::min<long long>((vs + 255) / 256, 128));      // blocks per sample
-    const int gb = std::max(1, std::min((g.Vh + 127) / 128, std::max(1, 4 * num_sms() / chunk)));
-    const int cb = (int)std::min<long long>((long long)chunk * ((g.Vh + CORR_SITES - 1) / CORR_SITES), 4 * num_sms());
-    double* dots = (double*)workspace(h, "ptc.dots", sizeof(double) * 4 * (size_t)n);
-    double* dpart = (double*)workspace(h, "ptc.dpart", sizeof(double) * 4 * (size_t)rb * chunk);
-    float* cpart = (float*)workspace(h, "ptc.cpart", sizeof(float) * (size_t)CORR_FLOATS * cb);
-    float* c0part = (float*)workspace(h, "ptc.c0part", sizeof(float) * 32 * (size_t)gb * chunk);
-    float* C = (float*)workspace(h, "ptc.C", sizeof(float) * (CORR_FLOATS + 32));
-    if (!m || !am || !t1 || !t2 || !gv || !phi || !dots || !dpart || !cpart || !c0part || !C)
-        return fail(h, WD_ERR_CUDA, "out of device memory");
+    uint4 *m, *am, *t1, *t2, *gv, *phi;
+    double *dots, *dpart;
+    float *cpart, *c0part, *C;
+    int gb = 0, cb = 0;
+    const int chunk = largest_chunk(
+        want,
+        [&](int c) {
+            m = (uint4*)workspace(h, "ptc.vm", vb * c);
+            am = (uint4*)workspace(h, "ptc.vam", vb * c);
+            t1 = (uint4*)workspace(h, "ptc.vt1", vb * c);
+            t2 = (uint4*)workspace(h, "ptc.vt2", vb * c);
+            gv = (uint4*)workspace(h, "ptc.vg", vb * c);
+            phi = (uint4*)workspace(h, "ptc.phi32", vb * 8 * c);
+            gb = std::max(1, std::min((g.Vh + 127) / 128, std::max(1, 4 * num_sms() / c)));
+            cb = (int)std::min<long long>((long long)c * ((g.Vh + CORR_SITES - 1) / CORR_SITES), 4 * num_sms());
+            dots = (double*)workspace(h, "ptc.dots", sizeof(double) * 4 * (size_t)n);
+            dpart = (double*)workspace(h, "ptc.dpart", sizeof(double) * 4 * (size_t)rb * c);
+            cpart = (float*)workspace(h, "ptc.cpart", sizeof(float) * (size_t)CORR_FLOATS * cb);
+            c0part = (float*)workspace(h, "ptc.c0part", sizeof(float) * 32 * (size_t)gb * c);
+            C = (float*)workspace(h, "ptc.C", sizeof(float) * (CORR_FLOATS + 32));
+            return m && am && t1 && t2 && gv && phi && dots && dpart && cpart && c0part && C;
+        },
+        [&]() {
+            for (const char* name : {"ptc.vm", "ptc.vam", "ptc.vt1", "ptc.vt2", "ptc.vg", "ptc.phi32"}) drop_workspace(h, name);
+            cudaGetLastError();   // the failed allocation's
+        });
+    if (chunk == 0) return fail(h, WD_ERR_CUDA, "out of device memory");
     static bool attr = false;
     if (!attr) {
         WD_CUDA(h, cudaFuncSetAttribute(k_ptc_corr, cudaFuncAttributeMaxDynamicSharedMemorySize, CORR_SMEM));
