@@ -99,7 +99,12 @@ template <typename T> constexpr int vec_block() { return sizeof(T) == 8 ? 64 : V
 // the kernel without look-ahead takes 128. With a clover block (even-odd
 // operator, two hops): FP16 21.4 26.3 - 58.0 against 16.0 24.7 - 61.7 without
 // look-ahead, BF16 22.5 28.0 - 62.5 against 14.9 23.3 - 63.2 (on FP32x2 pairs).
-// FP32 storage and the clover hops run 1-2% faster in blocks of 64 threads.
+// Blocks of 64 threads for FP32 storage and the hops with a clover block, 128 for the others (us with 128 / with 64):
+//   Vh                                   65536        120960       331776       1048576
+//   FP32, 12-real, plain hop           6.65 / 6.59  12.15 / 12.02  28.20 / 27.65  91.05 / 89.82
+//   FP32, 18-real, plain hop           7.93 / 7.92  13.61 / 13.46  34.65 / 34.36  112.96 / 112.61
+//   clover, FP16, even-odd operator   16.31 / 16.32 24.81 / 24.73  57.50 / 57.21  167.5 / 166.4
+//   clover, FP32, even-odd operator   17.15 / 17.24 34.40 / 34.18  92.20 / 91.58  268.3 / 267.0
 constexpr int FEW_SITES = 160000;
 template <typename T, int R> int default_variant(const Geom& g) {
     if (std::is_same<T, __nv_bfloat16>::value) return g.Vh <= FEW_SITES ? 1 : R == 12 ? 6 : 4;
