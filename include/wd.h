@@ -351,10 +351,10 @@ int wd_vec_axpby(wd_handle* h, int prec, const double a[2], const void* x, const
 /* Result of wd_tune. */
 typedef struct {
     int variant;          /* plain hop: kernel variant chosen (see wd_tune)                */
-    int block;            /* plain hop: threads per block chosen                           */
+    int block;            /* plain hop: threads per block chosen (fewer on small lattices)  */
     double us;            /* plain hop: its average launch time, microseconds              */
-    double default_us;    /* plain hop: the default configuration (variant 4, 128 threads) */
-    int candidates;       /* configurations timed per form                                 */
+    double default_us;    /* plain hop: what runs without wd_tune on this lattice          */
+    int candidates;       /* configurations considered per form (equal launches timed once) */
     int variant_reducing; /* hop with fused epilogue and dot products: variant chosen      */
     int block_reducing;   /* ... threads per block chosen                                  */
     double us_reducing;   /* ... its average launch time, microseconds                     */
@@ -379,13 +379,15 @@ typedef struct {
  * every candidate kernel variant and block size on scratch vectors (2 warm-up
  * and 8 timed launches each, CUDA events on `stream`) and keeps the fastest
  * for every later wd_apply / wd_solve / wd_solve_batch of the handle in that
- * (prec, recon); captured solver graphs are rebuilt. Candidates:
+ * (prec, recon); captured solver graphs are rebuilt. Candidates: what runs
+ * without wd_tune (WD_HOP_KERNEL and WD_HOP_BLOCK, else by lattice size), and
  * variant 4 (one site per thread, loads one direction ahead; 64 and 128
  * threads, and 256 except for FP16), 1 (no look-ahead), 2 (two sites per
  * thread, FP32x2; not FP64),
  * and for 16-bit storage 3 (tiles staged in shared memory), 6 (FP32x2 column
  * pairs; 64, 128 threads, and 256 for BF16) and, with 12-real links, 5 (per-thread cp.async
- * ring). These are the kernels of FP32 arithmetic. With wd_set_arith(16) and
+ * ring); the fixed-point FP64 hop has one kernel, of 64 or 128 threads. These
+ * are the kernels of FP32 arithmetic. With wd_set_arith(16) and
  * FP16 storage the FP16-arithmetic kernel runs instead (128 threads, one site
  * per thread); for nrhs > 1 wd_tune then also times it with K right-hand
  * sides per thread (every divisor K of nrhs up to 12; the site's 8 links are

@@ -169,7 +169,6 @@ __device__ __forceinline__ void rebuild_fixed(int mu, bool fwd, const long long 
     }
 }
 
-constexpr int HOP64_THREADS = 128;
 // Resident blocks per SM: 4 (128 registers). 3 (168 registers) is 2% faster at 32^3 x 64 (425 against 435 us), but at
 // 16^3 x 32 it leaves 56 of the 512 blocks to a second wave.
 constexpr int HOP64_BLOCKS = 4;

@@ -78,6 +78,8 @@ int spinor_units(int prec);
 // (vs64 for FP64 vectors), st = state array, g = guard kind.
 template <typename T> struct Ops {
     static cudaError_t hop(int recon, int epi, int red, const HopParams& P, cudaStream_t s);
+    // variant and threads per block of a hop whose HopParams choose none (environment, else by rule)
+    static void default_hop(int recon, const Geom& g, bool reducing, int* variant, int* block);
     // rev: order of the sites (sweep_site)
     static cudaError_t pupdate(int n, int nrhs, long long vs, uint4* p, const uint4* v, const uint4* r,
                                const SolverState* st, int rev, cudaStream_t s);
@@ -112,6 +114,22 @@ template <typename T> struct Ops {
 
 cudaError_t launch_unitarity(int nlinks, const double* U, unsigned long long* out, cudaStream_t s);
 
+int num_sms();
+inline int stream_blocks(int n, int block) {
+    long g = ((long)n + block - 1) / block;
+    return g < 1 ? 1 : (int)g;
+}
+
+// Threads per block of a launch over n items for each of nrhs right-hand sides: `block`, or on a small lattice a
+// half, quarter, ... of it down to one warp until every SM has a block. A kernel of 16 blocks of 128 threads (8^4)
+// otherwise runs on 16 of the 152 SMs.
+inline int spread_block(int n, int nrhs, int block) {
+    while (block > 32 && (long)stream_blocks(n, block) * nrhs < num_sms()) block /= 2;
+    return block;
+}
+
+constexpr int HOP64_THREADS = 128;   // largest block of the fixed-point FP64 hop
+
 // Block size of every vector kernel. The hop kernels take theirs from
 // HopParams::block (set by wd_tune), else from the environment (WD_HOP_BLOCK =
 // 64 or 128), else by rule (default_block).
@@ -130,6 +148,5 @@ int hop_variant();   // the environment's, 0 = none
 // Directions ahead that the FP16-arithmetic hop loads its neighbour spinors
 // (environment WD_HOP16_AHEAD = 1 or 2, default 2: 3% faster at 32^3 x 64).
 int hop16_ahead();
-int num_sms();
 
 }  // namespace wd

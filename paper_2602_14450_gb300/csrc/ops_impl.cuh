@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdlib>
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -69,19 +70,6 @@ inline int reduce_blocks(const void* kernel, int n, int block, int nrhs) {
     if (g > need) g = need;
     if (g > MAX_RED_BLOCKS) g = MAX_RED_BLOCKS;
     return g < 1 ? 1 : (int)g;
-}
-
-inline int stream_blocks(int n, int block) {
-    long g = ((long)n + block - 1) / block;
-    return g < 1 ? 1 : (int)g;
-}
-
-// Threads per block of a launch over n items for each of nrhs right-hand sides: `block`, or on a small lattice a
-// half, quarter, ... of it down to one warp until every SM has a block. A kernel of 16 blocks of 128 threads (8^4)
-// otherwise runs on 16 of the 152 SMs.
-inline int spread_block(int n, int nrhs, int block) {
-    while (block > 32 && (long)stream_blocks(n, block) * nrhs < num_sms()) block /= 2;
-    return block;
 }
 
 // Threads per block of the solver's vector kernels. In FP64 an SM works through its sites at the rate of its FP64
@@ -161,13 +149,13 @@ cudaError_t run_hop16m(const HopParams& Q, int K, cudaStream_t s) {
     return launch_k(hop16m_kernel<R, E, D, LSM>, nb * groups, blk, smem, s, Q);
 }
 
-// The FP64 hop in fixed point (SU(3) links). wd_tune's block size applies up to the kernel's 128 threads; the
+// The FP64 hop in fixed point (SU(3) links). A chosen block size applies up to the kernel's 128 threads; the
 // kernel variants are those of the floating-point hop and do not.
 template <int E, int D, bool MAT>
 cudaError_t run_hop64(const HopParams& P, cudaStream_t s) {
     constexpr int form = D == RED_NONE ? 0 : 1;
-    const int block = spread_block(P.g.Vh, P.nrhs, P.block[form] > 0 && P.block[form] < HOP64_THREADS
-                                                       ? P.block[form] : HOP64_THREADS);
+    const int want = P.block[form] > 0 ? P.block[form] : hop_block() ? hop_block() : HOP64_THREADS;
+    const int block = spread_block(P.g.Vh, P.nrhs, std::min(want, HOP64_THREADS));
     const void* k = (const void*)hop64_kernel<E, D, MAT>;
     const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, block) : reduce_blocks(k, P.g.Vh, block, P.nrhs);
     const cudaError_t e = launch_k(hop64_kernel<E, D, MAT>, nb * P.nrhs, block, 0, s, P);
@@ -293,6 +281,12 @@ cudaError_t run_hop(const HopParams& P, cudaStream_t s) {
     const int nb = (D == RED_NONE) ? stream_blocks(P.g.Vh, block) : reduce_blocks(k, P.g.Vh, block, nr);
     { const cudaError_t le_ = launch_k(hop_kernel<T, R, E, D, false>, nb * nr, block, 0, s, P); if (le_ != cudaSuccess) return le_; }
     return cudaGetLastError();
+}
+
+template <typename T>
+void Ops<T>::default_hop(int recon, const Geom& g, bool reducing, int* variant, int* block) {
+    *variant = hop_variant() ? hop_variant() : recon == 12 ? default_variant<T, 12>(g) : default_variant<T, 18>(g);
+    *block = hop_block() ? hop_block() : default_block<T>(reducing);
 }
 
 template <typename T>

@@ -2,6 +2,7 @@
 // timing every candidate on this lattice (CUDA events on the caller's stream),
 // separately for the plain hop and for the hop with fused epilogue and dot
 // products that ends every even-odd operator of the inner solve.
+#include <algorithm>
 #include <vector>
 
 #include "handle.h"
@@ -68,9 +69,26 @@ extern "C" int wd_tune(wd_handle* h, int prec, int recon, int nrhs, void* stream
     const std::vector<Cand> cands = candidates(prec, recon);
     Cand best[2] = {cands[0], cands[0]};
     float best_ms[2] = {1e30f, 1e30f}, default_ms = 0.f;
+    int considered = 0;
     cudaError_t err = cudaSuccess;
     for (int form = 0; form < 2 && err == cudaSuccess; ++form) {
-        for (const Cand& c : cands) {
+        Cand def{0, 0};
+        by_prec(prec, [&](auto tag) {
+            typedef typename decltype(tag)::type T;
+            Ops<T>::default_hop(recon, h->g, form == 1, &def.variant, &def.block);
+            return cudaSuccess;
+        });
+        std::vector<Cand> list{def}, timed;   // the default first; a launch that two candidates share is timed once
+        list.insert(list.end(), cands.begin(), cands.end());
+        considered = 0;
+        for (const Cand& c : list) {
+            if (&c == &list[0] || c.variant != def.variant || c.block != def.block) ++considered;
+            const Cand launched = P.fixed64 ? Cand{0, spread_block(h->g.Vh, nrhs, std::min(c.block, HOP64_THREADS))}
+                                            : Cand{c.variant, spread_block(h->g.Vh, nrhs, c.block)};
+            if (std::any_of(timed.begin(), timed.end(), [&](const Cand& o) {
+                    return o.variant == launched.variant && o.block == launched.block; }))
+                continue;
+            timed.push_back(launched);
             P.variant[form] = c.variant;
             P.block[form] = c.block;
             auto launch = [&]() {
@@ -89,7 +107,7 @@ extern "C" int wd_tune(wd_handle* h, int prec, int recon, int nrhs, void* stream
             if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
             if (err != cudaSuccess) break;
             ms /= 8.f;
-            if (form == 0 && c.variant == 4 && c.block == 128) default_ms = ms;
+            if (form == 0 && timed.size() == 1) default_ms = ms;
             if (ms < best_ms[form]) {
                 best_ms[form] = ms;
                 best[form] = c;
@@ -160,7 +178,7 @@ extern "C" int wd_tune(wd_handle* h, int prec, int recon, int nrhs, void* stream
         out->block = best[0].block;
         out->us = 1e3 * best_ms[0];
         out->default_us = 1e3 * default_ms;
-        out->candidates = (int)cands.size();
+        out->candidates = considered;
         out->variant_reducing = best[1].variant;
         out->block_reducing = best[1].block;
         out->us_reducing = 1e3 * best_ms[1];
