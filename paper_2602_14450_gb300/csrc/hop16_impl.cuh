@@ -164,8 +164,9 @@ __device__ __forceinline__ void reconstruct16(int mu, bool fwd, unsigned fb, con
 // multiply and FMA (one complex number per float2): the half2 accumulator is
 // widened and unscaled pairwise and out = a H + b y (+ c z) is formed with the
 // same per-lane roundings as the scalar epilogue, then rounded to FP16 and
-// stored. The dot products of the stored values are the scalar epilogue's
-// expressions term for term, so every result has the scalar epilogue's bits.
+// stored; the stored values have the scalar epilogue's bits. Their dot products
+// are chains of fused multiply-adds (add_fused), rounded once less per pair
+// than the scalar epilogue's.
 template <int EPI, int RED>
 __device__ __forceinline__ void epilogue16x2(const HopParams& P, uint4* vout, const uint4* vy, const uint4* vz,
                                              const uint4* vrs, int h, const __half2 (&acc)[12], float unscale,

@@ -22,7 +22,9 @@ template <typename C> __device__ __forceinline__ void sub_products(C& s, C a, C 
 template <> __device__ __forceinline__ void sub_products<double>(double& s, double a, double b, double c, double d) {
     s = fma(-c, d, fma(a, b, s));
 }
-// The same as two fused multiply-adds in FP32 (the dot products of the FP16-arithmetic hop).
+// The same as two fused multiply-adds in FP32 (the dot products of the FP16-arithmetic hop): two roundings instead of
+// three and two operations instead of three. One inner iteration of the FP16-mixed solve at 32^3 x 64: 931.1 us with
+// the expressions above, 926.6 us so; at 24^3 x 48 376.4 and 375.6 us (three runs each, within 1.3 us).
 __device__ __forceinline__ void add_fused(float& s, float a, float b, float c, float d) { s = fma(c, d, fma(a, b, s)); }
 __device__ __forceinline__ void sub_fused(float& s, float a, float b, float c, float d) { s = fma(-c, d, fma(a, b, s)); }
 
