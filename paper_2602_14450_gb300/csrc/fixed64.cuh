@@ -109,8 +109,6 @@ __host__ __device__ __forceinline__ Fixed signed_by(Fixed a, int mask) {
     a.neg ^= mask;
     return a;
 }
-__host__ __device__ __forceinline__ long long value(Fixed a) { return (long long)(a.v + (unsigned)-a.neg); }
-
 __host__ __device__ __forceinline__ long long sum(Fixed a, Fixed b) {
     return (long long)(a.v + b.v + (unsigned)-(a.neg + b.neg));
 }

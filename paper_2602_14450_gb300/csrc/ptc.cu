@@ -294,9 +294,7 @@ __global__ void __launch_bounds__(128, 5) k_ptc_s2_pf(Geom g, const uint4* in_e,
 }
 
 // Second pass on the even sites x: M psi(x) = V[0][0] psi(x) + sum_d T_{1+d} phi_{1+d}(x).
-// CMAJOR: phi units are colour-major (unit a = spins 0..3 of colour a, as the
-// tensor-core first pass writes them); otherwise the spinor order of load_spinor.
-template <typename TIN, typename TPHI, typename TOUT, typename LT, int R, bool CMAJOR>
+template <typename TIN, typename TPHI, typename TOUT, typename LT, int R>
 __global__ void __launch_bounds__(128) k_ptc_s2(Geom g, const uint4* in_e, const uint4* phi, long long pvs,
                                                 uint4* out_e, const uint4* links_e, const float2* V,
                                                 const SolverState* guard) {
@@ -319,18 +317,7 @@ __global__ void __launch_bounds__(128) k_ptc_s2(Geom g, const uint4* in_e, const
             bool wrap;
             const int hn = neighbour(g, h, co, d, &wrap);
             float m[18], t[24];
-            if constexpr (CMAJOR) {
-                constexpr int NU = Unit<TPHI>::N;
-                static_assert(NU == 8, "colour-major phi holds 8 reals per unit");
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const uint4 w = __ldg(phi + (size_t)d * pvs + (size_t)a * g.Vh + hn);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) f[2 * (3 * (e >> 1) + a) + (e & 1)] = Unit<TPHI>::get(w, e);
-                }
-            } else {
-                load_spinor<TPHI>(phi + (size_t)d * pvs, g.Vh, hn, f);
-            }
+            load_spinor<TPHI>(phi + (size_t)d * pvs, g.Vh, hn, f);
             load_link<LT, R>(links_e, g.Vh, h, d, m);
             colour_mul(m, f, t);
             const float ph = (wrap && g.bc[d >> 1] < 0) ? -1.f : 1.f;
@@ -695,7 +682,7 @@ static cudaError_t ptc_apply_f32(wd_handle* h, int n, const uint4* in_e, uint4* 
     const long long pvs = (long long)spinor_units(WD_FP32) * g.Vh;
     k_ptc_s1<float, float, float, 18><<<dim3((int)std::min(groups, cap), n), 128, 0, s>>>(g, in_e, PHI, pvs, lo, V,
                                                                                           guard);
-    k_ptc_s2<float, float, float, float, 18, false><<<dim3(grid_for(g.Vh, 128), n), 128, 0, s>>>(
+    k_ptc_s2<float, float, float, float, 18><<<dim3(grid_for(g.Vh, 128), n), 128, 0, s>>>(
         g, in_e, PHI, pvs, out_e, le, V, guard);
     return cudaGetLastError();
 }
@@ -727,7 +714,7 @@ cudaError_t ptc_apply_m(wd_handle* h, int prec, const uint4* in_e, uint4* out_e,
     } else {
         const long long pvs = (long long)spinor_units(WD_BF16) * g.Vh;
         k_ptc_s1<__half, __nv_bfloat16, __half, 12><<<g1, 128, 0, s>>>(g, in_e, PHI, pvs, lo, V, guard);
-        k_ptc_s2<__half, __nv_bfloat16, __half, __half, 12, false><<<g2, 128, 0, s>>>(g, in_e, PHI, pvs, out_e, le, V,
+        k_ptc_s2<__half, __nv_bfloat16, __half, __half, 12><<<g2, 128, 0, s>>>(g, in_e, PHI, pvs, out_e, le, V,
                                                                                         guard);
     }
     return cudaGetLastError();
