@@ -509,10 +509,10 @@ static int apply_n(wd_handle* h, int prec, int recon, int op, int nrhs, const vo
         if (cf_e) {   // out = C in first, then the hop adds to it in place
             e = by_prec(prec, [&](auto tag) {
                 typedef typename decltype(tag)::type T;
-                cudaError_t r2 = Ops<T>::apply_chiral(h->g.Vh, nrhs, 2 * vsu, cf_e, (const uint4*)ie, (uint4*)oe, s);
+                cudaError_t r2 = Ops<T>::apply_chiral(h->g.Vh, nrhs, 2 * vsu, cf_e, (const uint4*)ie, (uint4*)oe, true, s);
                 if (r2 == cudaSuccess)
                     r2 = Ops<T>::apply_chiral(h->g.Vh, nrhs, 2 * vsu, cf_o, (const uint4*)(ie + half),
-                                           (uint4*)(oe + half), s);
+                                           (uint4*)(oe + half), true, s);
                 return r2;
             });
             ye = oe;

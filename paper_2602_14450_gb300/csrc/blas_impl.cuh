@@ -477,10 +477,10 @@ __global__ void __launch_bounds__(256) k_rescale_in(int n, int nrhs, long long v
     grid_reduce<2, ST_INIT>(v, rc, sl);
 }
 
-// out = M in site by site with M in the chiral packing
+// out = M in, or with `one` in + M in, site by site with M in the chiral packing
 template <typename T>
 __global__ void __launch_bounds__(256) k_apply_chiral(int n, int nrhs, long long vs, const uint4* mat,
-                                                      const uint4* in, uint4* out) {
+                                                      const uint4* in, uint4* out, bool one) {
     typedef typename Unit<T>::C C;
     const Slice sl = slice_of(nrhs);
     in += sl.rhs * vs;
@@ -489,6 +489,10 @@ __global__ void __launch_bounds__(256) k_apply_chiral(int n, int nrhs, long long
         C v[24], o[24];
         load_spinor<T>(in, n, h, v);
         mat_mul_chiral<T>(mat, n, h, v, o);
+        if (one) {
+#pragma unroll
+            for (int i = 0; i < 24; ++i) o[i] += v[i];
+        }
         store_spinor<T>(out, n, h, o);
     }
 }

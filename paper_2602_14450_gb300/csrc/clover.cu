@@ -4,15 +4,19 @@
 //   sigma_mu_nu = (i/2) [gamma_mu, gamma_nu],
 //   Fh_mu_nu = traceless part of (Q_mu_nu - Q_mu_nu^+) / (8 i),
 // Q_mu_nu(x) the four plaquettes of the mu-nu plane with a corner at x, each
-// traversed mu-then-nu. Built once per gauge field; C and C^-1 are stored in
-// FP64 in the chiral packing (two Hermitian 6 x 6 blocks, 80 reals per site;
-// see mat_mul_chiral), other precisions are made from it on first use.
+// traversed mu-then-nu. Built once per gauge field; C - 1 and C^-1 are stored
+// in FP64 in the chiral packing (two Hermitian 6 x 6 blocks, 80 reals per site;
+// see mat_mul_chiral), other precisions are made from it on first use. C - 1
+// rather than C, since the packing forms the elements that connect opposite
+// chiralities as differences of the two blocks' elements: with the 1 in them
+// they would be held to the rounding of 1.
 //
 // In the chiral combinations the spin matrices are Pauli matrices:
 // sigma_ij = -eps_ijk sigma_k and sigma_k4 = -(off-diagonal) sigma_k, so block
 // c (sg = -1, +1) is
-//   S = 1/2 + (c_sw kappa / 2) sum_k sigma_k (x) G_k,   G = (F_12 + sg F_03, -F_02 + sg F_13, F_01 + sg F_23)
-// (directions 0..3 = x, y, z, t), and the packing of C^-1 is S^-1 / 4.
+//   S = 1/2 + T,   T = (c_sw kappa / 2) sum_k sigma_k (x) G_k,   G = (F_12 + sg F_03, -F_02 + sg F_13, F_01 + sg F_23)
+// (directions 0..3 = x, y, z, t), the packing of
+// C - 1 is T and that of C^-1 is S^-1 / 4.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -263,8 +267,8 @@ __global__ void __launch_bounds__(192) k_clover_build(Geom g, Field f, double ck
     double s[36];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        s[i] = 0.5 + gz[i];
-        s[3 + i] = 0.5 - gz[i];
+        s[i] = gz[i];
+        s[3 + i] = -gz[i];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             // (a, b) element of G: diagonal real, upper triangle stored, lower its conjugate
@@ -288,6 +292,8 @@ __global__ void __launch_bounds__(192) k_clover_build(Geom g, Field f, double ck
         }
     }
     store_chiral(p == 0 ? fwd_e : fwd_o, g.Vh, h, warp, s);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) s[i] += 0.5;
     double r[36];
 #pragma unroll
     for (int i = 0; i < 36; ++i) r[i] = s[i];
@@ -344,7 +350,7 @@ int clover_build(wd_handle* h) {
     return WD_OK;
 }
 
-// Clover blocks of kind 0 (C^{-1}) or 1 (C) in precision prec (chiral packing)
+// Clover blocks of kind 0 (C^{-1}) or 1 (C - 1) in precision prec (chiral packing)
 // for both parities; null pointers when the handle has no clover term.
 int ensure_clover(wd_handle* h, int prec, int kind, const uint4** even, const uint4** odd) {
     *even = *odd = nullptr;

@@ -62,7 +62,7 @@ struct wd_handle {
 
     double csw = 0.0;                  // clover coefficient of wd_set_clover (0: plain Wilson)
     bool have_clover = false;
-    uint4* clov64[2][2] = {};          // clover blocks [C^-1, C][parity] in FP64, chiral packing, of the gauge field
+    uint4* clov64[2][2] = {};          // clover blocks [C^-1, C - 1][parity] in FP64, chiral packing, of the gauge field
     uint4* clov[2][4][2] = {};         // the blocks an operator of a precision uses, made from them on first use
 
     // hop kernel chosen by wd_tune per [prec][recon 12 -> 0, 18 -> 1][without / with fused reduction]; 0 = default
@@ -100,7 +100,7 @@ RedCtx red_ctx(wd_handle* h, int stage);
 // h->herr once their stream has been synchronised.
 int* lower_err(wd_handle* h);
 // Clover blocks (clover.cu): rebuild from the gauge field; fetch kind 0 (C^-1)
-// or 1 (C) in a precision (null pointers without a clover term).
+// or 1 (C - 1) in a precision (null pointers without a clover term).
 int clover_build(wd_handle* h);
 int ensure_clover(wd_handle* h, int prec, int kind, const uint4** even, const uint4** odd);
 // 1 + 12 |c_sw| kappa bounds the norm of every clover block C.

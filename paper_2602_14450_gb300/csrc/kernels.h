@@ -102,9 +102,9 @@ template <typename T> struct Ops {
     // xo = eta + kappa t and the sum of |eta - xo + kappa t|^2 (Eq. 5 with t = H_oe xi_e)
     static cudaError_t odd_reconstruct(int n, int nrhs, long long vs, double kappa, const uint4* eta, const uint4* t,
                                        uint4* xo, RedCtx rc, cudaStream_t s);
-    // out = M in with M in the chiral packing (80 reals per site, see mat_mul_chiral)
+    // out = M in, or with `one` in + M in, with M in the chiral packing (80 reals per site, see mat_mul_chiral)
     static cudaError_t apply_chiral(int n, int nrhs, long long vs, const uint4* mat, const uint4* in, uint4* out,
-                                    cudaStream_t s);
+                                    bool one, cudaStream_t s);
     // chiral packing in storage T from FP64
     static cudaError_t chiral_from64(int n, const uint4* src64, uint4* dst, cudaStream_t s);
     static cudaError_t pack(const Geom& g, int parity, const double* lex, uint4* out, cudaStream_t s);

@@ -310,8 +310,8 @@ cudaError_t Ops<T>::hop(int recon, int epi, int red, const HopParams& P, cudaStr
 
 template <typename T>
 cudaError_t Ops<T>::apply_chiral(int n, int nrhs, long long vs, const uint4* mat, const uint4* in, uint4* out,
-                                 cudaStream_t s) {
-    k_apply_chiral<T><<<stream_blocks(n, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, mat, in, out);
+                                 bool one, cudaStream_t s) {
+    k_apply_chiral<T><<<stream_blocks(n, VEC_BLOCK) * nrhs, VEC_BLOCK, 0, s>>>(n, nrhs, vs, mat, in, out, one);
     return cudaGetLastError();
 }
 
