@@ -231,6 +231,12 @@ __device__ __forceinline__ void store_chiral(uint4* dst, int Vh, int h, int c, c
     }
 }
 
+// Largest real of F below which a plane's products are formed in FP64 arithmetic also for SU(3) links. FP64 arithmetic
+// holds F to 2e-16 of its largest element whatever its size (the imaginary parts of near-unit links are products with
+// one small factor), fixed point to 2e-18 absolute times a few: 2e-17 of F at 0.3, 6e-17 at 0.1, 2e-16 at 0.03, 6e-15
+// at 1e-3 (rms over random links).
+constexpr double WEAK_FIELD = 0.0625;
+
 // One block takes 32 sites of one parity (blockIdx.y): each of its six warps
 // forms the field strength of one plane, then warps 0 and 1 assemble and
 // invert one chiral block each. Bound: in FP64 arithmetic the products (6480
@@ -249,7 +255,13 @@ __global__ void __launch_bounds__(192) k_clover_build(Geom g, Field f, double ck
         const int mu = warp < 3 ? 0 : warp < 5 ? 1 : 2;
         const int nu = warp < 3 ? warp + 1 : warp < 5 ? warp - 1 : 3;
         double t[9];
-        plane_field<FIXED>(g, f, coord_of(g, p, h), mu, nu, t);
+        const Coord c = coord_of(g, p, h);
+        plane_field<FIXED>(g, f, c, mu, nu, t);
+        if (FIXED) {   // a weak field is smaller than the products it is left over from: FP64 arithmetic
+            double most = 0.0;
+            for (int i = 0; i < 9; ++i) most = fmax(most, fabs(t[i]));
+            if (most < WEAK_FIELD) plane_field<false>(g, f, c, mu, nu, t);
+        }
         const double tr = (t[0] + t[1] + t[2]) / 3.0;
         for (int i = 0; i < 9; ++i) F[warp][i][lane] = i < 3 ? t[i] - tr : t[i];
     }

@@ -34,3 +34,14 @@ def test_storage_precision_of_weak_fields(prec, j):
     dims = (4, 4, 4, 6)
     got, want = off_diagonal(synth.gauge_random(dims, 0.02, seed=9), 1.0, 0.12, dims, prec, j)
     assert (got - want).abs().amax() <= 8 * ROUND[prec] * want.abs().amax()
+
+
+# Links within eps of 1. A real of F is a sum over four leaves of products of four links of which one factor is small, 16
+# such terms: at most 22 roundings of 16 eps, and F itself is of size eps. 0.3 and 0.03: on both sides of the border
+# between fixed point and FP64 arithmetic.
+@pytest.mark.parametrize("eps", [0.3, 0.03, 1e-3, 1e-5, 1e-8])
+@pytest.mark.parametrize("j", [0, 4, 8, 11])
+def test_fp64_blocks_of_weak_fields(eps, j):
+    dims = (2, 4, 4, 6)
+    got, want = off_diagonal(synth.gauge_random(dims, eps, seed=9), 1.0, 0.12, dims, "fp64", j)
+    assert (got - want).abs().amax() <= 22 * 16 * 1.1e-16 * want.abs().amax()
