@@ -29,8 +29,9 @@
 // below; SIZE_MIN is that in its units of 2^(E-1032). On rough links 1 site in
 // 10^6 fails; components fed by small spinor parts or small link entries alone do,
 // and reals that are zero.
-// The relative error of a hop of Gaussian fields is 0.92e-16 against 1.0e-16
-// in FP64 arithmetic.
+// The relative error of a hop of Gaussian fields is 0.50e-16 against 1.42e-16
+// in FP64 arithmetic (tests/test_gpu_fixed64_exact.py), of D_W, with its
+// epilogue in FP64, 0.92e-16 against 1.0e-16.
 //
 // Bounds (rows of unit norm, |h| < 2^60): |sum u1 h0| <= sqrt(6) 2^29 2^31 and
 // |sum u0 h1| <= 6 2^31 2^28, together 6.3e18 < 2^63; a product is at most

@@ -138,6 +138,27 @@ def lex(psi):
     return synth.to_host_layout(psi).cuda()
 
 
+def test_relative_error_of_gaussian_fields_is_that_of_fp64_arithmetic():
+    """Relative L2 error of a hop (the figure in csrc/fixed64.cuh), in fixed point and, with links scaled off SU(3), in
+    FP64 arithmetic; run with -s to print them."""
+    dims, bc = (4, 2, 4, 4), (1, 1, 1, -1)
+    u, psi = fields(dims, "gauss")
+    err = []
+    for links in (u, u * (1.0 + 1e-5)):
+        lat = lattice(links, 0.1, dims, bc)
+        src, dst = packed(lat, "fp64"), packed(lat, "fp64")
+        lat.pack("fp64", 1, lex(psi), src)
+        lat.apply("fp64", 18, wd.WD_OP_HOP_EO, src, dst)
+        got = torch.zeros_like(lex(psi))
+        lat.unpack("fp64", 0, dst, got)
+        got = got.cpu().reshape(-1, 24).tolist()
+        want = exact_hop(links, psi, 0, bc)
+        num = sum((F(got[s][i]) - v) ** 2 for s, r in want.items() for i, (v, _) in enumerate(r))
+        err.append((float(num) / float(sum(v * v for r in want.values() for v, _ in r))) ** 0.5)
+    print("relative L2 error: fixed point %.3e, FP64 arithmetic %.3e" % tuple(err))
+    assert err[0] <= err[1] <= 2e-16
+
+
 @pytest.mark.parametrize("dims,split", [((2, 2, 4, 4), (3,)), ((4, 2, 2, 6), (0, 3)), ((2, 4, 4, 2), (1, 2))])
 def test_split_hop_takes_its_scale_from_its_own_neighbours(dims, split):
     """Interior hop of a sub-lattice whose field is larger on one face: the sites of the opposite face, whose hops
