@@ -13,9 +13,12 @@
 // One CTA takes 128 odd sites: its 128 threads compute the transports (one site
 // each, FP32 arithmetic) and write them, rounded to BF16, as three M = 128 x
 // K = 64 operand tiles (one per colour); one thread issues the MMAs
-// (M = 128, N = 64, 4 x K = 16 per colour) into 64 TMEM columns; each warp reads
-// its 32 rows back (tcgen05.ld) and stores phi colour-major: unit a of field d2
-// holds (s = 0..3, re/im) of colour a.
+// (M = 128, N = 64, 4 x K = 16 per colour); each warp reads its 32 rows back
+// (tcgen05.ld) and stores phi colour-major: unit a of field d2 holds
+// (s = 0..3, re/im) of colour a. Colours 0 and 1 are issued together into two
+// 64-column accumulators and colour 2 follows into the first as soon as it has
+// been read, so a tile waits for the tensor core once and synchronises three
+// times (one accumulator, a wait and two barriers per colour: @@BEFORE@@).
 //
 // Operand layout in shared memory: the no-swizzle K-major canonical form of
 // 8-row x 16-byte core matrices. Element (m, k) of a tile with K = 64 sits at
@@ -38,7 +41,7 @@ constexpr int K = 64, N = 64;                // real K and N of the contraction
 constexpr int A_TILE_BYTES = TILE_M * K * 2; // one colour's operand tile (16 KB)
 constexpr int B_BYTES = N * K * 2;           // 8 KB
 constexpr int SMEM_BYTES = 3 * A_TILE_BYTES + B_BYTES + 64;
-constexpr int TMEM_COLS = 64;
+constexpr int TMEM_COLS = 128;              // two accumulators; three CTAs an SM take 384 of its 512 columns
 constexpr unsigned WAIT_LIMIT = 1u << 22;    // try_wait rounds before giving up (the default)
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -97,14 +100,18 @@ __device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity, unsigne
     return false;
 }
 
-// 8 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// 32 consecutive FP32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+    uint32_t r[32];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                  : "r"(taddr));
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 
@@ -130,7 +137,7 @@ __global__ void __launch_bounds__(128, 3) k_ptc_s1_tc(Geom g, const uint4* in_e,
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* A = smem;                              // 3 colour tiles
     unsigned char* B = smem + 3 * A_TILE_BYTES;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(B + B_BYTES);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(B + B_BYTES);   // one per accumulator
     uint32_t* tslot = reinterpret_cast<uint32_t*>(B + B_BYTES + 16);
     const int tid = threadIdx.x, warp = tid >> 5;
 
@@ -145,6 +152,7 @@ __global__ void __launch_bounds__(128, 3) k_ptc_s1_tc(Geom g, const uint4* in_e,
     }
     if (tid == 0) {
         bar_init(bar, 1);
+        bar_init(bar + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 0) {
@@ -160,8 +168,31 @@ __global__ void __launch_bounds__(128, 3) k_ptc_s1_tc(Geom g, const uint4* in_e,
     const uint32_t tmem = *tslot;
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     const uint32_t a_base = smem_addr(A), b_base = smem_addr(B);
-    uint32_t phase = 0;
+    uint32_t issued[2] = {0, 0};   // commits on each barrier so far; the last one completes the phase of parity (n - 1) & 1
     bool failed = false;
+    auto issue = [&](int a) {      // colour a into accumulator a & 1
+        if (tid == 0) {
+#pragma unroll
+            for (int j = 0; j < K / 16; ++j) {
+                const uint64_t ad = smem_desc(a_base + a * A_TILE_BYTES + 256 * j, 128, 1024);
+                const uint64_t bd = smem_desc(b_base + 256 * j, 128, 1024);
+                tc::mma_bf16(tmem + 64 * (a & 1), ad, bd, j > 0 ? 1u : 0u);
+            }
+            mma_commit(bar + (a & 1));
+        }
+        ++issued[a & 1];
+    };
+    // waits for an accumulator's last MMA and reads this thread's row of it; false when the wait ran out in this warp
+    auto read = [&](int acc, float (&v)[64]) {
+        const bool landed = __all_sync(0xffffffffu, bar_wait(bar + acc, (issued[acc] - 1) & 1, limit));
+        if (landed) {
+            fence_after();
+            tmem_ld32(tmem + lane_base + 64 * acc, v);
+            tmem_ld32(tmem + lane_base + 64 * acc + 32, v + 32);
+            tmem_ld_wait();
+        }
+        return landed;
+    };
 
     const int ntiles = (g.Vh + TILE_M - 1) / TILE_M;
     for (int tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
@@ -218,46 +249,41 @@ __global__ void __launch_bounds__(128, 3) k_ptc_s1_tc(Geom g, const uint4* in_e,
         __syncthreads();
         fence_after();
 
-#pragma unroll 1
-        for (int a = 0; a < 3; ++a) {
-            if (tid == 0) {
-#pragma unroll
-                for (int j = 0; j < K / 16; ++j) {
-                    const uint64_t ad = smem_desc(a_base + a * A_TILE_BYTES + 256 * j, 128, 1024);
-                    const uint64_t bd = smem_desc(b_base + 256 * j, 128, 1024);
-                    tc::mma_bf16(tmem, ad, bd, j > 0 ? 1u : 0u);
-                }
-                mma_commit(bar);
-            }
-            const bool landed = bar_wait(bar, phase, limit);
-            failed = __syncthreads_or(!landed);     // uniform across the CTA
-            if (failed) {                           // `phase` stays the one still pending
-                if (tid == 0 && err) *(volatile int*)err = 1;
-                break;
-            }
-            phase ^= 1;
-            fence_after();
-            // every lane takes part in the aligned TMEM loads; rows past the end are not stored
+        auto store = [&](int a, const float (&v)[64]) {   // rows past the end are not stored
+            if (!ok) return;
 #pragma unroll
             for (int d2 = 0; d2 < 8; ++d2) {
-                float v[8];
-                tmem_ld8(tmem + lane_base + 8 * d2, v);
-                tmem_ld_wait();
-                if (ok) {
-                    uint4 w;
-                    w.x = pack_bf16(v[0], v[1]);
-                    w.y = pack_bf16(v[2], v[3]);
-                    w.z = pack_bf16(v[4], v[5]);
-                    w.w = pack_bf16(v[6], v[7]);
-                    phi[(size_t)d2 * pvs + (size_t)a * g.Vh + h] = w;
-                }
+                uint4 w;
+                w.x = pack_bf16(v[8 * d2], v[8 * d2 + 1]);
+                w.y = pack_bf16(v[8 * d2 + 2], v[8 * d2 + 3]);
+                w.z = pack_bf16(v[8 * d2 + 4], v[8 * d2 + 5]);
+                w.w = pack_bf16(v[8 * d2 + 6], v[8 * d2 + 7]);
+                phi[(size_t)d2 * pvs + (size_t)a * g.Vh + h] = w;
             }
+        };
+        issue(0);
+        issue(1);
+        float row[64];
+        bool landed = read(0, row);
+        fence_before();
+        failed = __syncthreads_or(!landed);      // uniform across the CTA: accumulator 0 has been read
+        fence_after();
+        if (!failed) {
+            issue(2);
+            store(0, row);
+            landed = read(1, row);
+            if (landed) store(1, row);
+            const bool last = read(0, row);
+            if (last) store(2, row);
             fence_before();
-            __syncthreads();
+            failed = __syncthreads_or(!landed || !last);   // all read, and the operand tiles are free again
             fence_after();
         }
+        if (failed && tid == 0 && err) *(volatile int*)err = 1;
     }
-    if (failed && tid == 0) bar_wait(bar, phase);   // default bound: let an MMA still in flight finish
+    if (failed && tid == 0) {   // default bound: let MMAs still in flight finish
+        for (int i = 0; i < 2; ++i) bar_wait(bar + i, (issued[i] - 1) & 1);
+    }
     fence_before();
     __syncthreads();
     fence_after();
