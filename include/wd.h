@@ -182,8 +182,9 @@ int wd_gauge_unitarity(wd_handle* h, double* max_unitarity_dev, double* max_det_
  * hopping operators WD_OP_HOP_* are unchanged); the refinement stops when
  * |b^ - A xi_e| <= tol |eta| / (1 + 12 |c_sw| kappa), which bounds the full
  * residual |eta - D_sw xi| = |C_ee (b^ - A xi_e)| by tol |eta|. C and C^-1
- * are computed in FP64 on the device (Gauss-Jordan per site) and converted
- * to other precisions on first use; wd_set_gauge rebuilds them. c_sw = 0
+ * are computed in FP64 on the device (elimination per site) and converted
+ * to other precisions on first use; wd_set_gauge rebuilds them. Both calls
+ * wait for the device before they rewrite blocks. c_sw = 0
  * removes the term. Not available with WD_MIXED_FP16_LEARNED. Requires
  * wd_set_gauge first (WD_ERR_NO_GAUGE); WD_ERR_INVALID_ARG for a non-finite
  * c_sw or a singular block. */

@@ -242,8 +242,8 @@ constexpr double WEAK_FIELD = 0.0625;
 // invert one chiral block each. Bound: in FP64 arithmetic the products (6480
 // multiply-adds per site) keep the FP64 pipe busy; in fixed point they take the
 // integer multiplier a quarter of that time, and the inverses (~1000 FP64
-// operations) are half of the rest. Measured at 24^3 x 48: 3.3 ms, against
-// 53.7 ms with one thread per site and 12 x 12 blocks in local memory.
+// operations) are half of the rest. Measured at 24^3 x 48: 3.6 ms (3.3 without
+// the weak planes in FP64 arithmetic), against 53.7 ms with one thread per site and 12 x 12 blocks in local memory.
 template <bool FIXED>
 __global__ void __launch_bounds__(192) k_clover_build(Geom g, Field f, double ck, uint4* fwd_e, uint4* fwd_o,
                                                       uint4* inv_e, uint4* inv_o, int* singular) {

@@ -169,18 +169,21 @@ __device__ __forceinline__ void rebuild_fixed(int mu, bool fwd, const long long 
     }
 }
 
-// Resident blocks per SM: 4 (128 registers). 3 (168 registers) is 2% faster at 32^3 x 64 (425 against 435 us), but at
-// 16^3 x 32 it leaves 56 of the 512 blocks to a second wave.
+// Resident blocks per SM: 4 (128 registers). Before the size test 3 (168 registers) was 2% faster at 32^3 x 64 (425
+// against 435 us), but at 16^3 x 32 it leaves 56 of the 512 blocks to a second wave.
 constexpr int HOP64_BLOCKS = 4;
 
-// Bounds: a warp issues about 7500 instructions per 32 sites, 1728 of them
-// wide integer multiply-adds, which occupy the multiplier pipe 4.4-5.7 cycles
-// each (measured; 2.1 for other integer multiply-adds): ~0.3 of the 0.425 ms
-// at 32^3 x 64; the 1.6 GB of links and vectors take 0.24 ms. The same hop in
-// FP64 arithmetic (hop_kernel<double, 18>) takes 1.437 ms, all of it FP64 pipe.
+// Bounds: 491 us at 32^3 x 64, where the same hop in FP64 arithmetic
+// (hop_kernel<double, 18>) takes 1437, all of it FP64 pipe. A warp issues about
+// 9600 instructions per 32 sites, 1728 of them wide integer multiply-adds: the
+// multiplier pipe is busy 58% of the time and the schedulers 51%, at 15 warps
+// per SM waiting on results and loads (profiles/hop64_clover_corr.md). The 1.7
+// GB that it moves take 0.25 ms. The size test is 56 us of it, the exponent
+// without a spare binade 10.
 //
 // The eight directions run as one loop body rather than unrolled: unrolled,
-// the straight-line code ran at the rate of the instruction cache (770 us).
+// the straight-line code ran at the rate of the instruction cache (770 us,
+// against 435 without the size test, as the other figures here).
 // The spin structure is selected at run time: the partner spins of the
 // projection by the load addresses, the factor i by a selection of words,
 // signs by masks, and the rebuild by a branch that is the same for the whole
