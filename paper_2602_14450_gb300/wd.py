@@ -222,7 +222,8 @@ class Lattice:
     def set_gauge(self, u):
         """u: float64 tensor in the host layout [4, V, 3, 3, 2] (CPU or CUDA)."""
         where = WD_DEVICE if u.is_cuda else WD_HOST
-        self._check(lib().wd_set_gauge(self.h, _ptr(u.contiguous()), where), "wd_set_gauge")
+        u = u.contiguous()   # a copy has to outlive the call
+        self._check(lib().wd_set_gauge(self.h, _ptr(u), where), "wd_set_gauge")
 
     def set_clover(self, csw):
         """wd_set_clover: add the clover term with coefficient csw (0 removes it)."""
